@@ -80,7 +80,7 @@ k_adj_face(const Params prm, const double *__restrict__ lam, const double *__res
   constexpr int NT = NT_INVISCID;
   const OpsLayout L{P1, NP};
   __shared__ double s_op[4 * P1 * P1 + 3 * P1 + NP];
-  for (int t = threadIdx.x; t < L.size(); t += blockDim.x) s_op[t] = prm.ops[t];
+  for (int t = threadIdx.x; t < L.cf(); t += blockDim.x) s_op[t] = prm.ops[t];
   __syncthreads();
   const double *Dx = s_op + L.Dx(), *Dy = s_op + L.Dy();
   const double *invM = s_op + L.invM(), *wfx = s_op + L.wfx(), *wfy = s_op + L.wfy();

@@ -62,6 +62,7 @@ struct Params {
   double mu1, mu2, sigma, gx, gy;
   double Gamma, eps;
   double eta_x, eta_y;       // interior penalty on faces normal to x and to y
+  double dg, Ge, hdr, eta2_x, eta2_y;  // g1 - g2, Gamma eps, drho0 / 2, 2 eta
   int gravity, check_finite;
   int grad_lift;             // BR1-lifted gradients of phi and psi (dg_opts.grad_lift)
   const double *ops;         // operator tables, see OpsLayout
@@ -78,6 +79,11 @@ struct Params {
 //   invM[Np]     1 / (w_i w_j J)  (inverse of the collocated mass matrix)
 //   wfx [P1]     w_k * J_f on faces normal to x (1D: 1)
 //   wfy [P1]     w_k * J_f on faces normal to y
+//   cf  [2]      (w_k J_f) / 2 times invM at the face nodes: 1 / (w_0 hx) and 1 / (w_0 hy), the same
+//                for every k
+//   lw  [4][P1]  per face (W, E, S, N) and node c of a line normal to it: -1/2 (w_k J_f) invM times
+//                d l_c / dm at the face node, the weight with which the SIP flux's symmetric term
+//                reaches node c (again the same for every k)
 struct OpsLayout {
   int P1, Np;
   __host__ __device__ int Dx() const { return 0; }
@@ -88,7 +94,9 @@ struct OpsLayout {
   __host__ __device__ int invM() const { return 4 * P1 * P1 + P1; }
   __host__ __device__ int wfx() const { return 4 * P1 * P1 + P1 + Np; }
   __host__ __device__ int wfy() const { return 4 * P1 * P1 + 2 * P1 + Np; }
-  __host__ __device__ int size() const { return 4 * P1 * P1 + 3 * P1 + Np; }
+  __host__ __device__ int cf() const { return 4 * P1 * P1 + 3 * P1 + Np; }
+  __host__ __device__ int lw() const { return cf() + 2; }
+  __host__ __device__ int size() const { return lw() + 4 * P1; }
 };
 
 // Launch interface of one kernel family (one order, dimension and term set).
@@ -96,9 +104,7 @@ struct KernelSet {
   cudaError_t (*volume)(const Params &, const double *w, double *rvol, double *trace, cudaStream_t);
   cudaError_t (*surface)(const Params &, int mode, double dt, const double *w0, const double *ws,
                          const double *rvol, const double *trace, double *out, cudaStream_t);
-  int nt;       // trace fields per face node
-  int epb;      // elements per block
-  int threads;  // threads per block
+  int nt;  // trace fields per face node
 };
 
 // Kernel families by order (defined in dg_inst_p<P>.cu).

@@ -76,7 +76,8 @@ inline void lagrange_derivative_into(int n, const double *x, double *D) {
 
 // Operator table (OpsLayout, OpsLayout{p+1, Np}.size() doubles) for one
 // element size: (2/h) D, (2/h) Dhat with Dhat = W^-1 D^T W, the GLL weights,
-// the inverse of the collocated mass matrix and the face quadrature weights.
+// the inverse of the collocated mass matrix, the face quadrature weights and
+// the weights of face terms with M^-1 applied.
 inline void build_ops_into(int dim, int p, double hx, double hy, double *ops) {
   const int P1 = p + 1, Np = dim == 2 ? P1 * P1 : P1;
   const double J = dim == 2 ? 0.25 * hx * hy : 0.5 * hx;
@@ -103,6 +104,14 @@ inline void build_ops_into(int dim, int p, double hx, double hy, double *ops) {
     ops[L.wfx() + k] = dim == 2 ? wt[k] * 0.5 * hy : 1.0;
     ops[L.wfy() + k] = dim == 2 ? wt[k] * 0.5 * hx : 1.0;
   }
+  ops[L.cf()] = 1.0 / (wt[0] * hx);
+  ops[L.cf() + 1] = 1.0 / (wt[0] * hy);
+  for (int f = 0; f < 4; ++f)
+    for (int c = 0; c < P1; ++c) {
+      const int a = (f & 1) ? p : 0;  // the face's node on the line
+      const double h = f < 2 ? hx : hy, sg = (f & 1) ? 1.0 : -1.0;
+      ops[L.lw() + f * P1 + c] = -0.5 * sg * (2.0 / h) * D[a * P1 + c] * (2.0 / (h * wt[c]));
+    }
 }
 
 // Validation of one problem of the two-phase model: NULL when valid, else the
@@ -181,6 +190,11 @@ inline Params make_params(const dg_mesh *mesh, int p, const dg_eos *eos, double 
   q.eps = eps;
   q.eta_x = o.c_ip * P1 * P1 / hx;
   q.eta_y = o.c_ip * P1 * P1 / hy;
+  q.dg = q.g1 - q.g2;
+  q.Ge = Gamma * eps;
+  q.hdr = 0.5 * q.drho0;
+  q.eta2_x = 2.0 * q.eta_x;
+  q.eta2_y = 2.0 * q.eta_y;
   q.gravity = o.gravity != 0;
   q.check_finite = o.check_finite != 0;
   q.grad_lift = o.grad_lift != 0;

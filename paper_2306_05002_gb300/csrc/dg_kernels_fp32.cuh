@@ -719,7 +719,7 @@ __device__ __forceinline__ void surf32_body(const Params &prm, const ParamsF &pf
         e2_[fi] = act && t < NFK ? neighbour(prm, e, t / NK) : -1;
       }
     }
-    for (int t = threadIdx.x; t < L.size(); t += blockDim.x) s_op[t] = opsf[t];
+    for (int t = threadIdx.x; t < L.cf(); t += blockDim.x) s_op[t] = opsf[t];
     grid_dependency_wait();
   }
 
@@ -767,7 +767,7 @@ __device__ __forceinline__ void surf32_body(const Params &prm, const ParamsF &pf
   }
 
   if (!PDL)
-    for (int t = threadIdx.x; t < L.size(); t += blockDim.x) s_op[t] = opsf[t];
+    for (int t = threadIdx.x; t < L.cf(); t += blockDim.x) s_op[t] = opsf[t];
   __syncthreads();
   const float *Dx = s_op + L.Dx(), *Dy = s_op + L.Dy();
   const float *invM = s_op + L.invM(), *wfx = s_op + L.wfx(), *wfy = s_op + L.wfy();
@@ -1075,7 +1075,7 @@ cudaError_t launch_volume32(const Params &prm, const ParamsF &pf, const float *o
   const int blocks = (prm.E + G::EPB - 1) / G::EPB;
   static const int resident = resident_blocks(k_volume32<P, DIM, VISC, ST, true>, G::THREADS);
   if (blocks <= resident)
-    return launch_dependent(k_volume32<P, DIM, VISC, ST, true>, blocks, G::THREADS, s, prm, pf, opsf, w, rvol,
+    return launch_dependent(k_volume32<P, DIM, VISC, ST, true>, blocks, G::THREADS, 0, s, prm, pf, opsf, w, rvol,
                             trace, w64, w32out, lo_out, w64copy);
   k_volume32<P, DIM, VISC, ST, false><<<blocks, G::THREADS, 0, s>>>(prm, pf, opsf, w, rvol, trace, w64, w32out,
                                                                     lo_out, w64copy);
@@ -1089,7 +1089,7 @@ cudaError_t launch_surface32(const Params &prm, const ParamsF &pf, const float *
   const int blocks = (prm.E + G::EPB - 1) / G::EPB;
   static const int resident = resident_blocks(k_surface32<P, DIM, VISC, ST, true>, G::THREADS);
   if (blocks <= resident)
-    return launch_dependent(k_surface32<P, DIM, VISC, ST, true>, blocks, G::THREADS, s, prm, pf, opsf, mode,
+    return launch_dependent(k_surface32<P, DIM, VISC, ST, true>, blocks, G::THREADS, 0, s, prm, pf, opsf, mode,
                             dt, io, rvol, trace);
   k_surface32<P, DIM, VISC, ST, false><<<blocks, G::THREADS, 0, s>>>(prm, pf, opsf, mode, dt, io, rvol, trace);
   return cudaGetLastError();
@@ -1103,7 +1103,7 @@ cudaError_t launch_surfvol32(const Params &prm, const ParamsF &pf, const float *
   const int blocks = (prm.E + G::EPB - 1) / G::EPB;
   static const int resident = resident_blocks(k_surfvol32<P, DIM, VISC, ST, true>, G::THREADS);
   if (blocks <= resident)
-    return launch_dependent(k_surfvol32<P, DIM, VISC, ST, true>, blocks, G::THREADS, s, prm, pf, opsf, mode,
+    return launch_dependent(k_surfvol32<P, DIM, VISC, ST, true>, blocks, G::THREADS, 0, s, prm, pf, opsf, mode,
                             dt, io, rvol_in, tr_in, rvol_out, tr_out);
   k_surfvol32<P, DIM, VISC, ST, false><<<blocks, G::THREADS, 0, s>>>(prm, pf, opsf, mode, dt, io, rvol_in, tr_in,
                                                                      rvol_out, tr_out);

@@ -172,7 +172,7 @@ k_kin_stage(const KinParams kp, int mode, int kstep, double frac, const double *
   __shared__ double s_tr[EPB][NP][6];      // phi, psi, d(phi)/dx, d(phi)/dy, n_x, n_y
   __shared__ double s_surf[EPB][NFK][2];
   __shared__ double s_lift[EPB][NFK];
-  for (int t = threadIdx.x; t < L.size(); t += blockDim.x) s_op[t] = kp.ops[t];
+  for (int t = threadIdx.x; t < L.cf(); t += blockDim.x) s_op[t] = kp.ops[t];
   const double *Dx = s_op + L.Dx(), *Dy = s_op + L.Dy(), *Dhx = s_op + L.Dhx(), *Dhy = s_op + L.Dhy();
   const double *invM = s_op + L.invM(), *wfx = s_op + L.wfx(), *wfy = s_op + L.wfy();
 

@@ -37,7 +37,7 @@ unsigned char *g_noalloc_addr[kMaxDevices] = {};
 size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
 
 // The largest operator table (p = 5, 2D).
-constexpr int kMaxOps = 4 * HOST_MAXP1 * HOST_MAXP1 + 3 * HOST_MAXP1 + HOST_MAXP1 * HOST_MAXP1;
+constexpr int kMaxOps = 5 * HOST_MAXP1 * HOST_MAXP1 + 7 * HOST_MAXP1 + 2;
 struct OpsArg {
   double v[kMaxOps];
 };

@@ -39,11 +39,12 @@ inline int resident_blocks(K kernel, int threads) {
 
 // Launch with the programmatic-serialization attribute.
 template <typename... K, typename... A>
-inline cudaError_t launch_dependent(void (*kernel)(K...), int blocks, int threads, cudaStream_t s, A &&...args) {
+inline cudaError_t launch_dependent(void (*kernel)(K...), int blocks, int threads, size_t smem, cudaStream_t s,
+                                    A &&...args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(blocks);
   cfg.blockDim = dim3(threads);
-  cfg.dynamicSmemBytes = 0;
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

@@ -146,7 +146,7 @@ k_ri_surface(const ReinitParams rp, int mode, double dtau, const double *w0, con
   __shared__ double s_op[4 * P1 * P1 + 3 * P1 + NP];
   __shared__ double s_surf[EPB][NFK];
   __shared__ double s_lift[EPB][NFK];
-  for (int t = threadIdx.x; t < L.size(); t += blockDim.x) s_op[t] = rp.ops[t];
+  for (int t = threadIdx.x; t < L.cf(); t += blockDim.x) s_op[t] = rp.ops[t];
   __syncthreads();
   const double *Dx = s_op + L.Dx(), *Dy = s_op + L.Dy();
   const double *invM = s_op + L.invM(), *wfx = s_op + L.wfx(), *wfy = s_op + L.wfy();
