@@ -63,6 +63,7 @@ struct Params {
   double Gamma, eps;
   double eta_x, eta_y;       // interior penalty on faces normal to x and to y
   double dg, Ge, hdr, eta2_x, eta2_y;  // g1 - g2, Gamma eps, drho0 / 2, 2 eta
+  double Gp_x, Gp_y;                   // 2 Gamma eps eta
   int gravity, check_finite;
   int grad_lift;             // BR1-lifted gradients of phi and psi (dg_opts.grad_lift)
   const double *ops;         // operator tables, see OpsLayout

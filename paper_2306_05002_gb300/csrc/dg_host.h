@@ -195,6 +195,8 @@ inline Params make_params(const dg_mesh *mesh, int p, const dg_eos *eos, double 
   q.hdr = 0.5 * q.drho0;
   q.eta2_x = 2.0 * q.eta_x;
   q.eta2_y = 2.0 * q.eta_y;
+  q.Gp_x = q.Ge * q.eta2_x;
+  q.Gp_y = q.Ge * q.eta2_y;
   q.gravity = o.gravity != 0;
   q.check_finite = o.check_finite != 0;
   q.grad_lift = o.grad_lift != 0;

@@ -100,9 +100,8 @@ __device__ __forceinline__ double sg_pressure(const Params &p, double phi, doubl
 // large one the count that leaves the fewest idle lanes.  Ties go to the larger block (fewer
 // copies of the operator table).
 constexpr int MAX_THREADS64 = 192;
-template <int P, int DIM>
-inline int pick_epb64(int E, int cn, int cf) {
-  constexpr int NP = Geom<P, DIM, false, false>::NP, NFK = Geom<P, DIM, false, false>::NFK;
+// per: threads' tasks per element (its nodes); perf: face nodes.
+inline int pick_epb64(int E, int per, int cn, int perf = 0, int cf = 0) {
   static const int sms = [] {
     int dev = 0, n = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -111,11 +110,11 @@ inline int pick_epb64(int E, int cn, int cf) {
     return n;
   }();
   int best = 1;
-  double best_cost = 0.0;
-  for (int epb = 1; epb == 1 || (epb * NP + 31) / 32 * 32 <= MAX_THREADS64; ++epb) {
-    const int wn = (epb * NP + 31) / 32, wf = (epb * NFK + 31) / 32;
+  long best_cost = 0;
+  for (int epb = 1; epb == 1 || (epb * per + 31) / 32 * 32 <= MAX_THREADS64; ++epb) {
+    const int wn = (epb * per + 31) / 32, wf = (epb * perf + 31) / 32;
     const long blocks = (E + epb - 1) / epb;
-    const double cost = (double)((blocks + sms - 1) / sms) * (cn * wn + cf * wf);
+    const long cost = (blocks + sms - 1) / sms * (cn * wn + cf * wf);
     if (epb == 1 || cost <= best_cost) {
       best = epb;
       best_cost = cost;
@@ -130,8 +129,8 @@ inline int pick_epb64(int E, int cn, int cf) {
 // the time (64 x 64, p = 3: 191 us a step with an early trigger, 141 without).
 //
 // Bound by the FP64 pipe.  64 x 64, p = 3 in 2D: a step of three volume and three surface launches
-// 172 -> 141 us, of which shared reciprocals, integer comparisons and one face value per axis and
-// node 24 us, the update's inputs loaded ahead of the face work and the dependent launches 7 us.
+// 172 -> 141 us (loading the update's inputs ahead of the face work: no gain, and 3% slower where the
+// grid has several waves, for the registers it holds).
 template <int P, int DIM>
 __global__ void __launch_bounds__(MAX_THREADS64)
 k_volume(const Params prm, int epb, const double *__restrict__ w, double *__restrict__ rvol,
@@ -365,22 +364,6 @@ k_surface(const Params prm, int epb, int mode, double dt, const double *__restri
   const int N = prm.N;
   const long n = (long)e * NP + a;
   const bool act = le < epb && e < prm.E && in_bounds(prm.status, n, N);
-  // the node's inputs of the update, loaded ahead of the face work that hides their latency
-  double rv[NV], wn[NV], w0n[NV];
-#pragma unroll
-  for (int vv = 0; vv < NV; ++vv) rv[vv] = wn[vv] = w0n[vv] = 0.0;
-  if (act) {
-#pragma unroll
-    for (int vv = 0; vv < NV; ++vv) rv[vv] = __ldca(rvol + (long)vv * N + n);
-    if (mode != MODE_RHS) {
-#pragma unroll
-      for (int vv = 0; vv < NV; ++vv) wn[vv] = __ldca(ws + (long)vv * N + n);
-    }
-    if (mode == MODE_S2 || mode == MODE_S3) {
-#pragma unroll
-      for (int vv = 0; vv < NV; ++vv) w0n[vv] = __ldca(w0 + (long)vv * N + n);
-    }
-  }
   if (prm.dt_dev) dt = __ldca(prm.dt_dev);
 
   // Phase 1: numerical fluxes at the block's face nodes.  S and the terms below carry a factor two
@@ -526,11 +509,11 @@ k_surface(const Params prm, int epb, int mode, double dt, const double *__restri
 #pragma unroll
   for (int vv = 0; vv < NV; ++vv) {
     const long o = (long)vv * N + n;
-    double r = fma(acc[vv], im, rv[vv]);
+    double r = fma(acc[vv], im, __ldca(rvol + o));
     if (mode != MODE_RHS) {
-      r = fma(dt, r, wn[vv]);
-      if (mode == MODE_S2) r = fma(0.25, r, 0.75 * w0n[vv]);
-      else if (mode == MODE_S3) r = fma(2.0 / 3.0, r, (1.0 / 3.0) * w0n[vv]);
+      r = fma(dt, r, __ldca(ws + o));
+      if (mode == MODE_S2) r = fma(0.25, r, 0.75 * __ldca(w0 + o));
+      else if (mode == MODE_S3) r = fma(2.0 / 3.0, r, (1.0 / 3.0) * __ldca(w0 + o));
     }
     bad |= !finite64(r);
     out[o] = r;
@@ -541,7 +524,7 @@ k_surface(const Params prm, int epb, int mode, double dt, const double *__restri
 template <int P, int DIM>
 cudaError_t launch_volume(const Params &prm, const double *w, double *rvol, double *trace, cudaStream_t s) {
   using G = Geom<P, DIM, false, false>;
-  const int epb = pick_epb64<P, DIM>(prm.E, 1, 0), threads = (epb * G::NP + 31) / 32 * 32;
+  const int epb = pick_epb64(prm.E, G::NP, 1), threads = (epb * G::NP + 31) / 32 * 32;
   const size_t smem = sizeof(double) * (4 * G::P1 * G::P1 + (size_t)G::NSTAGE * epb * G::NP);
   return launch_dependent(k_volume<P, DIM>, (prm.E + epb - 1) / epb, threads, smem, s, prm, epb, w, rvol, trace);
 }
@@ -551,7 +534,7 @@ cudaError_t launch_surface(const Params &prm, int mode, double dt, const double 
                            const double *rvol, const double *trace, double *out, cudaStream_t s) {
   using G = Geom<P, DIM, false, false>;
   // a face node costs about as much as a node here
-  const int epb = pick_epb64<P, DIM>(prm.E, 1, 1), threads = (epb * G::NP + 31) / 32 * 32;
+  const int epb = pick_epb64(prm.E, G::NP, 1, G::NFK, 1), threads = (epb * G::NP + 31) / 32 * 32;
   const size_t smem =
       sizeof(double) * (2 * G::P1 * G::P1 + G::NP + 2 * NFT * G::P1 + (size_t)(NV + 6) * epb * G::NFK);
   return launch_dependent(k_surface<P, DIM>, (prm.E + epb - 1) / epb, threads, smem, s, prm, epb, mode, dt, w0, ws,

@@ -470,7 +470,7 @@ k_surface_full(const Params prm, int epb, int mode, double dt, const double *__r
 template <int P, bool VISC, bool ST>
 cudaError_t launch_volume_full(const Params &prm, const double *w, double *rvol, double *trace, cudaStream_t s) {
   using G = Geom<P, 2, VISC, ST>;
-  const int epb = pick_epb64<P, 2>(prm.E, 1, 0), threads = (epb * G::NP + 31) / 32 * 32;
+  const int epb = pick_epb64(prm.E, G::NP, 1), threads = (epb * G::NP + 31) / 32 * 32;
   const size_t smem = sizeof(double) * (4 * G::P1 * G::P1 + (size_t)G::NSTAGE * epb * G::NP);
   return launch_dependent(k_volume_full<P, VISC, ST>, (prm.E + epb - 1) / epb, threads, smem, s, prm, epb, w, rvol,
                           trace);
@@ -481,7 +481,7 @@ cudaError_t launch_surface_full(const Params &prm, int mode, double dt, const do
                            const double *rvol, const double *trace, double *out, cudaStream_t s) {
   using G = Geom<P, 2, VISC, ST>;
   // face nodes cost about as much as nodes here (46 and 50 operations)
-  const int epb = pick_epb64<P, 2>(prm.E, 1, 1), threads = (epb * G::NP + 31) / 32 * 32;
+  const int epb = pick_epb64(prm.E, G::NP, 1, G::NFK, 1), threads = (epb * G::NP + 31) / 32 * 32;
   const size_t smem = sizeof(double) * (2 + 4 * G::P1 + (size_t)NSP * epb * G::NFK);
   return launch_dependent(k_surface_full<P, VISC, ST>, (prm.E + epb - 1) / epb, threads, smem, s, prm, epb, mode, dt,
                           w0, ws, rvol, trace, out);
