@@ -406,8 +406,8 @@ dg_status dg_kin_step(dg_ctx *ctx, double *w, double t0, double dt, int nsteps, 
    min(0.5 h / (2p + 1), 0.1 h^2 / ((2p + 1)^2 nu)), h the smallest element
    width.  The paper applies ~50 iterations every 2000 steps.  FP64; works on
    FP64 and FP32-bulk contexts alike (on the FP64 state).  The first call
-   allocates the context's re-initialisation workspace (4 N doubles and the
-   face traces), kept until dg_destroy.  Rectangles only: a triangle context
+   allocates the context's re-initialisation workspace (3 N doubles and two
+   sets of face traces), kept until dg_destroy.  Rectangles only: a triangle context
    gives DG_ERR_UNSUPPORTED.  Asynchronous on stream. */
 dg_status dg_reinit(dg_ctx *ctx, double *w, int niter, double nu, double dtau, void *stream);
 

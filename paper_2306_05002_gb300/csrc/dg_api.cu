@@ -249,9 +249,10 @@ struct dg_ctx {
   TriKernels tk{};
   int tri_grid = 0;
   double *d_kacc = nullptr, *d_kwsA = nullptr, *d_kwsB = nullptr;
-  double *d_kt0 = nullptr, *d_kxi = nullptr, *d_ktv = nullptr;
+  double *d_kt = nullptr, *d_kxi = nullptr, *d_ktv = nullptr;
+  double *d_krvol = nullptr, *d_ktr = nullptr;  // rectangles: volume part, two buffers of face traces
   // level-set re-initialisation workspace (dg_reinit), allocated on first use
-  double *d_riS = nullptr, *d_ri1 = nullptr, *d_ri2 = nullptr, *d_rirvol = nullptr, *d_ritr = nullptr;
+  double *d_riS = nullptr, *d_ri1 = nullptr, *d_rirvol = nullptr, *d_ritr = nullptr;
   double *d_part = nullptr, *d_diag = nullptr;
   unsigned *d_status = nullptr;
   int nparts = 0;
@@ -275,12 +276,13 @@ struct dg_ctx {
     const double *states = nullptr, *tapes = nullptr, *lam = nullptr;
   } seg[2];
   const double *g_w = nullptr;
-  double *d_dt = nullptr;      // the step size the captured dg_step / dg_kin_step graphs read
+  double *d_dt = nullptr;      // the step size the captured dg_step graphs read
   double dt_set = 0.0;         // the value last written there (0: none)
   std::string err = "no error";
 };
 
 static const int GRAPH_UNROLL = 8;
+static_assert(GRAPH_UNROLL <= KIN_MAX_STEPS, "stage time factors of a captured sequence");
 static_assert(GRAPH_UNROLL <= (int)(sizeof(dg_ctx::StepGraphs::grem) / sizeof(cudaGraphExec_t)),
               "remainder graph slots");
 
@@ -335,8 +337,8 @@ static void free_ctx(dg_ctx *c) {
   cudaFree(c->d_ops);
   cudaFree(c->d_hstate);
   cudaFree(c->d_copy64);
-  for (double *q : {c->d_kacc, c->d_kwsA, c->d_kwsB, c->d_kt0, c->d_kxi, c->d_ktv}) cudaFree(q);
-  for (double *q : {c->d_riS, c->d_ri1, c->d_ri2, c->d_rirvol, c->d_ritr}) cudaFree(q);
+  for (double *q : {c->d_kacc, c->d_kwsA, c->d_kwsB, c->d_kt, c->d_kxi, c->d_ktv, c->d_krvol, c->d_ktr}) cudaFree(q);
+  for (double *q : {c->d_riS, c->d_ri1, c->d_rirvol, c->d_ritr}) cudaFree(q);
   cudaFree(c->d_w1);
   cudaFree(c->d_w2);
   cudaFree(c->d_rvol);
@@ -1217,7 +1219,7 @@ extern "C" dg_status dg_batch_step(dg_ctx *c, double *const *w, const double *dt
 // ---------------------------------------------------------------------------
 
 namespace dgpf {
-__global__ void k_kin_set_time(double *t0, double t);
+__global__ void k_kin_set_time(KinParams kp, double *kt, double t, double dt);
 }
 
 extern "C" dg_status dg_kin_create(const dg_mesh *mesh, int p, double Gamma, double eps, const dg_velocity *vel,
@@ -1280,6 +1282,9 @@ extern "C" dg_status dg_kin_create(const dg_mesh *mesh, int p, double Gamma, dou
   k.eps = eps;
   k.eta_x = cip * c->P1 * c->P1 / c->hx;
   k.eta_y = cip * c->P1 * c->P1 / c->hy;
+  k.Ge = Gamma * eps;
+  k.Gp_x = 2.0 * k.Ge * k.eta_x;
+  k.Gp_y = 2.0 * k.Ge * k.eta_y;
   k.eta_tri = cip * (p + 1) * (p + 2);
   if (tri) tri_constants(c->hx, c->hy, k.eta_tri, k.tc);
   k.vel = vel->kind;
@@ -1298,10 +1303,16 @@ extern "C" dg_status dg_kin_create(const dg_mesh *mesh, int p, double Gamma, dou
   gll_nodes(p, xi, wt);
   const size_t sb = c->len * sizeof(double);
   cudaError_t e = cudaSuccess;
-  // one kernel per stage on either element type: no volume residual or face traces in memory
-  double **bufs[] = {&c->d_kacc, &c->d_kwsA, &c->d_kwsB};
-  for (double **b : bufs)
-    if (e == cudaSuccess) e = cudaMalloc(b, sb);
+  // triangles: one kernel per stage and two stage inputs; rectangles: the volume part and the face
+  // traces of the next stage instead
+  e = cudaMalloc(&c->d_kacc, sb);
+  if (tri) {
+    if (e == cudaSuccess) e = cudaMalloc(&c->d_kwsA, sb);
+    if (e == cudaSuccess) e = cudaMalloc(&c->d_kwsB, sb);
+  } else {
+    if (e == cudaSuccess) e = cudaMalloc(&c->d_krvol, sb);
+    if (e == cudaSuccess) e = cudaMalloc(&c->d_ktr, (size_t)2 * KIN_NT * c->E * c->NFK * sizeof(double));
+  }
   // the velocity's spatial factor at every node (rectangles) or quadrature point (triangles)
   const size_t vrows = tri ? (size_t)c->E * c->tk.points : (size_t)c->N;
   if (e == cudaSuccess) e = cudaMalloc(&c->d_ktv, 2 * vrows * sizeof(double));
@@ -1313,15 +1324,13 @@ extern "C" dg_status dg_kin_create(const dg_mesh *mesh, int p, double Gamma, dou
     const long groups = (c->E + tri_group(p) - 1) / tri_group(p);
     c->tri_grid = (int)std::max(1L, std::min(groups, (long)std::max(1, sms) * std::max(1, per_sm)));
   }
-  if (e == cudaSuccess) e = cudaMalloc(&c->d_kt0, sizeof(double));
-  if (e == cudaSuccess) e = cudaMalloc(&c->d_dt, sizeof(double));
-  if (e == cudaSuccess) e = cudaMemset(c->d_dt, 0, sizeof(double));  // dg_kin_rhs: stage time t0 exactly
+  if (e == cudaSuccess) e = cudaMalloc(&c->d_kt, KT_SIZE * sizeof(double));
   if (e == cudaSuccess) e = cudaMalloc(&c->d_kxi, xi.size() * sizeof(double));
   if (e == cudaSuccess) e = cudaMalloc(&c->d_ops, ops.size() * sizeof(double));
   if (e == cudaSuccess) e = cudaMalloc(&c->d_status, sizeof(unsigned));
   if (e == cudaSuccess) e = cudaMemcpy(c->d_ops, ops.data(), ops.size() * sizeof(double), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(c->d_kxi, xi.data(), xi.size() * sizeof(double), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemset(c->d_kt0, 0, sizeof(double));
+  if (e == cudaSuccess) e = cudaMemset(c->d_kt, 0, KT_SIZE * sizeof(double));
   if (e == cudaSuccess) e = cudaMemset(c->d_status, 0, sizeof(unsigned));
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking);
   if (e != cudaSuccess) {
@@ -1332,8 +1341,7 @@ extern "C" dg_status dg_kin_create(const dg_mesh *mesh, int p, double Gamma, dou
   }
   k.ops = c->d_ops;
   k.xi = c->d_kxi;
-  k.t0 = c->d_kt0;
-  k.dt = c->d_dt;
+  k.kt = c->d_kt;
   k.status = c->d_status;
   k.vel_tab = c->d_ktv;
   e = tri ? c->tk.velocity_table(k, c->d_ktv, c->cap) : c->kk.velocity_table(k, c->d_ktv, c->cap);
@@ -1396,43 +1404,45 @@ extern "C" dg_status dg_kin_rhs(dg_ctx *c, const double *w, double t, double *L,
   if (r != DG_OK) return r;
   if (!w || !L || w == L) return fail(c, DG_ERR_ARG, "dg_kin_rhs: need distinct, non-null w and L");
   cudaStream_t s = (cudaStream_t)stream;
-  k_kin_set_time<<<1, 1, 0, s>>>(c->d_kt0, t);
+  k_kin_set_time<<<1, 4 * KIN_MAX_STEPS, 0, s>>>(c->kp, c->d_kt, t, 0.0);
   cudaError_t e = cudaGetLastError();
   if (c->tri) {
-    if (e == cudaSuccess) e = c->tk.stage(c->kp, KIN_RHS, 0, 0.0, w, nullptr, nullptr, L, c->tri_grid, s);
+    if (e == cudaSuccess) e = c->tk.stage(c->kp, KIN_RHS, 0, w, nullptr, nullptr, L, c->tri_grid, s);
     return e == cudaSuccess ? DG_OK : cuda_fail(c, e, "dg_kin_rhs: launch");
   }
-  if (e == cudaSuccess) e = c->kk.stage(c->kp, KIN_RHS, 0, 0.0, w, nullptr, nullptr, L, s);
+  if (e == cudaSuccess) e = c->kk.volume(c->kp, 0, w, c->d_krvol, c->d_ktr, s);
+  if (e == cudaSuccess)
+    e = c->kk.stage(c->kp, KIN_RHS, 0, true, nullptr, nullptr, c->d_krvol, c->d_ktr, nullptr, L, s);
   return e == cudaSuccess ? DG_OK : cuda_fail(c, e, "dg_kin_rhs: launch");
 }
 
-// One classical RK4 step of the captured sequence: step k of the graph, stage
-// inputs w -> A -> B -> A, the last stage writes w in place.  The kernels read
-// the step size from device memory (c->d_dt) and form the stage times there.
-static dg_status enqueue_kin_step(dg_ctx *c, double *w, int k, cudaStream_t s) {
+// `steps` classical RK4 steps of the captured sequence.  The kernels read the step size and the stage
+// times' velocity factors from device memory (c->d_kt), stage st of step k at index 4 k + st.
+// Rectangles: the volume part of the first stage, then one launch per stage that leaves the volume
+// part and the traces of the next one; the trace buffers alternate.  Triangles: stage inputs
+// w -> A -> B -> A, the last stage writes w in place.
+static dg_status enqueue_kin_steps(dg_ctx *c, double *w, int steps, cudaStream_t s) {
+  const int mode[4] = {KIN_K1, KIN_K2, KIN_K3, KIN_K4};
   double *A = c->d_kwsA, *B = c->d_kwsB;
-  const double frac[4] = {0.0, 0.5, 0.5, 1.0};
   const double *in[4] = {w, A, B, A};
   double *out[4] = {A, B, A, w};
-  const int mode[4] = {KIN_K1, KIN_K2, KIN_K3, KIN_K4};
-  for (int st = 0; st < 4; ++st) {
-    cudaError_t e;
-    if (c->tri) {
-      e = c->tk.stage(c->kp, mode[st], k, frac[st], in[st], w, c->d_kacc, out[st], c->tri_grid, s);
-    } else {
-      e = c->kk.stage(c->kp, mode[st], k, frac[st], in[st], w, c->d_kacc, out[st], s);
-    }
-    if (e != cudaSuccess) return cuda_fail(c, e, "dg_kin_step: launch");
+  const size_t half = (size_t)KIN_NT * c->E * c->NFK;
+  cudaError_t e = c->tri ? cudaSuccess : c->kk.volume(c->kp, 0, w, c->d_krvol, c->d_ktr, s);
+  for (int q = 0; q < 4 * steps && e == cudaSuccess; ++q) {
+    if (c->tri)
+      e = c->tk.stage(c->kp, mode[q & 3], q, in[q & 3], w, c->d_kacc, out[q & 3], c->tri_grid, s);
+    else
+      e = c->kk.stage(c->kp, mode[q & 3], q, q == 4 * steps - 1, w, c->d_kacc, c->d_krvol, c->d_ktr + (q & 1) * half,
+                      c->d_ktr + (~q & 1) * half, w, s);
   }
-  return DG_OK;
+  return e == cudaSuccess ? DG_OK : cuda_fail(c, e, "dg_kin_step: launch");
 }
 
 static dg_status capture_kin(dg_ctx *c, double *w, int steps, cudaGraphExec_t *exec) {
   cudaGraph_t g = nullptr;
   cudaError_t e = cudaStreamBeginCapture(c->cap, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) return cuda_fail(c, e, "dg_kin_step: begin capture");
-  dg_status r = DG_OK;
-  for (int k = 0; k < steps && r == DG_OK; ++k) r = enqueue_kin_step(c, w, k, c->cap);
+  const dg_status r = enqueue_kin_steps(c, w, steps, c->cap);
   e = cudaStreamEndCapture(c->cap, &g);
   if (r != DG_OK) {
     if (g) cudaGraphDestroy(g);
@@ -1458,15 +1468,10 @@ extern "C" dg_status dg_kin_step(dg_ctx *c, double *w, double t0, double dt, int
   }
   cudaStream_t s = (cudaStream_t)stream;
   cudaError_t e = cudaSuccess;
-  if (dt != c->dt_set) {
-    k_set_double<<<1, 1, 0, s>>>(c->d_dt, dt);
-    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(c, e, "dg_kin_step: set dt");
-    c->dt_set = dt;
-  }
   int done = 0;
   while (done < nsteps && e == cudaSuccess) {
     const bool big = nsteps - done >= GRAPH_UNROLL;
-    k_kin_set_time<<<1, 1, 0, s>>>(c->d_kt0, t0 + done * dt);
+    k_kin_set_time<<<1, 4 * KIN_MAX_STEPS, 0, s>>>(c->kp, c->d_kt, t0 + done * dt, dt);
     e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaGraphLaunch(big ? c->gk : c->g1, s);
     done += big ? GRAPH_UNROLL : 1;
@@ -1494,8 +1499,8 @@ extern "C" dg_status dg_reinit(dg_ctx *c, double *w, int niter, double nu, doubl
     rp.N = c->kp.N;
     for (int f = 0; f < 4; ++f) rp.bc[f] = BC_PERIODIC;
     rp.eps = c->kp.eps;
-    rp.eta_x = c->kp.eta_x;
-    rp.eta_y = c->kp.eta_y;
+    rp.eta2_x = 2.0 * c->kp.eta_x;
+    rp.eta2_y = 2.0 * c->kp.eta_y;
   } else {
     rp.nx = c->prm.nx;
     rp.ny = c->prm.ny;
@@ -1503,8 +1508,8 @@ extern "C" dg_status dg_reinit(dg_ctx *c, double *w, int niter, double nu, doubl
     rp.N = c->prm.N;
     for (int f = 0; f < 4; ++f) rp.bc[f] = c->prm.bc[f];
     rp.eps = c->prm.eps;
-    rp.eta_x = c->prm.eta_x;
-    rp.eta_y = c->prm.eta_y;
+    rp.eta2_x = c->prm.eta2_x;
+    rp.eta2_y = c->prm.eta2_y;
   }
   rp.ops = c->d_ops;
   rp.status = c->d_status;
@@ -1514,13 +1519,13 @@ extern "C" dg_status dg_reinit(dg_ctx *c, double *w, int niter, double nu, doubl
   if (!(dtau > 0.0)) dtau = std::min(0.5 * h / q, 0.1 * h * h / (q * q * rp.nu));
   cudaError_t e = cudaSuccess;
   if (!c->d_riS) {
-    const size_t nb = (size_t)rp.N * sizeof(double), tb = (size_t)2 * rp.E * rk.nfk * sizeof(double);
-    double **bufs[] = {&c->d_riS, &c->d_ri1, &c->d_ri2, &c->d_rirvol};
+    const size_t nb = (size_t)rp.N * sizeof(double), tb = (size_t)4 * rp.E * rk.nfk * sizeof(double);
+    double **bufs[] = {&c->d_riS, &c->d_ri1, &c->d_rirvol};
     for (double **b : bufs)
       if (e == cudaSuccess) e = cudaMalloc(b, nb);
     if (e == cudaSuccess) e = cudaMalloc(&c->d_ritr, tb);
     if (e != cudaSuccess) {
-      for (double **b : {&c->d_riS, &c->d_ri1, &c->d_ri2, &c->d_rirvol, &c->d_ritr}) {
+      for (double **b : {&c->d_riS, &c->d_ri1, &c->d_rirvol, &c->d_ritr}) {
         cudaFree(*b);
         *b = nullptr;
       }
@@ -1532,14 +1537,14 @@ extern "C" dg_status dg_reinit(dg_ctx *c, double *w, int niter, double nu, doubl
   cudaStream_t s = (cudaStream_t)stream;
   double *psi = w + rp.N;
   e = rk.sign(rp, w, c->d_riS, s);
+  // one launch per stage after the first volume part; the two trace buffers alternate
   const int mode[3] = {MODE_S1, MODE_S2, MODE_S3};
-  const double *in[3] = {psi, c->d_ri1, c->d_ri2};
-  double *out[3] = {c->d_ri1, c->d_ri2, psi};
-  for (int it = 0; it < niter && e == cudaSuccess; ++it)
-    for (int st = 0; st < 3 && e == cudaSuccess; ++st) {
-      e = rk.volume(rp, in[st], c->d_riS, c->d_rirvol, c->d_ritr, s);
-      if (e == cudaSuccess) e = rk.surface(rp, mode[st], dtau, psi, in[st], c->d_rirvol, c->d_ritr, out[st], s);
-    }
+  const long long nst = 3LL * niter;
+  const size_t half = (size_t)2 * rp.E * rk.nfk;
+  if (e == cudaSuccess && niter > 0) e = rk.volume(rp, psi, c->d_riS, c->d_rirvol, c->d_ritr, s);
+  for (long long q = 0; q < nst && e == cudaSuccess; ++q)
+    e = rk.stage(rp, mode[q % 3], dtau, q == nst - 1, psi, c->d_ri1, c->d_riS, c->d_rirvol, c->d_ritr + (q & 1) * half,
+                 c->d_ritr + (~q & 1) * half, s);
   return e == cudaSuccess ? DG_OK : cuda_fail(c, e, "dg_reinit: launch");
 }
 

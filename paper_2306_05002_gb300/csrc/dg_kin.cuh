@@ -14,9 +14,10 @@
 // function interpolated at each element's nodes (discretely divergence-free,
 // normal components continuous across faces: the phase field's mass is then
 // conserved to round-off).  Time integration is the classical four-stage
-// Runge-Kutta method; each stage is one launch (k_kin_stage), which also
-// evaluates the neighbours' face traces from their nodal values.  Periodic
-// meshes only.
+// Runge-Kutta method: a volume launch on the state (k_kin_volume), then one
+// launch per stage (k_kin_stage: face fluxes from the traces, M^-1, the stage
+// update and the volume part of the next stage on the result, which the
+// thread of each node holds).  Periodic meshes only.
 #pragma once
 
 #include <math_constants.h>
@@ -44,6 +45,7 @@ struct KinParams {
   int nx, ny, E, N;
   double x0, y0, hx, hy;
   double Gamma, eps, eta_x, eta_y;
+  double Ge, Gp_x, Gp_y;   // Gamma eps, 2 Gamma eps eta
   int vel;                 // VEL_UNIFORM or VEL_RIDER_KOTHE
   double u0, v0, T;        // uniform velocity; Rider-Kothe period
   double xc, yc;           // Rider-Kothe vortex centre
@@ -53,8 +55,7 @@ struct KinParams {
                            // (triangles), see kin_velocity_factor
   const double *ops;       // operator table (OpsLayout)
   const double *xi;        // GLL nodes on [-1, 1]
-  const double *t0;        // device: time at the start of the captured step sequence
-  const double *dt;        // device: the step size of the captured step sequences
+  const double *kt;        // device: step sizes and time factors of the captured sequence (KinTime)
   int check_finite;
   unsigned *status;
 };
@@ -76,6 +77,13 @@ __device__ __forceinline__ void kin_velocity_factor(const KinParams &kp, double 
     *V = kp.v0;
   }
 }
+
+// What the stage kernels of a captured sequence read from device memory, set before every launch of
+// the sequence: dt/2, dt, dt/6 and the velocity's time factor c at every stage, stage st of step k
+// at index KT_C + 4 k + st.  A cosine in every block would cost half of a stage kernel's FP64 work.
+enum KinTime { KT_HALF = 0, KT_DT, KT_SIXTH, KT_C };
+constexpr int KIN_MAX_STEPS = 8;  // steps of the longest captured sequence
+constexpr int KT_SIZE = KT_C + 4 * KIN_MAX_STEPS;
 
 __device__ __forceinline__ double kin_time_factor(const KinParams &kp, double t) {
   return kp.vel == VEL_RIDER_KOTHE ? cos(CUDART_PI * t / kp.T) : 1.0;
@@ -140,217 +148,237 @@ __device__ __forceinline__ int kin_face_node(int f, int kk) {
   return f == 0 ? kk * P1 : (f == 1 ? P + kk * P1 : (f == 2 ? kk : kk + P * P1));
 }
 
-// One stage of the kinematic mode in one launch: broken gradients, n, a_1,
-// the volume term of -a_1 (D^ contractions) and the non-conservative
-// transport at every node; at every face node the transport flux
-// (lambda - m.u-) [[f]] and the SIP flux of a_1 with its lifted symmetric
-// term, the neighbour's trace being evaluated here from its nodal values (a
-// row of the neighbour's element), not read from a trace buffer; then M^-1
-// and the right-hand side or an RK4 stage:
-//   K1: acc = L,        out = w0 + dt/2 L
-//   K2: acc += 2 L,     out = w0 + dt/2 L
-//   K3: acc += 2 L,     out = w0 + dt L
-//   K4: out = w0 + dt/6 (acc + L)   (out may be w0: each node is read, then
-//                                    written, by the same thread)
-// Neighbour values come from the stage input, which no stage writes, so the
-// stages need no synchronisation beyond stream order.  The step size is read
-// from device memory (*kp.dt), so captured step sequences serve any dt; the
-// stage time is *kp.t0 + (kstep dt) + (frac dt), kstep the step's index in the
-// captured sequence and frac the stage's fraction of the step (0, 1/2, 1/2, 1).
+// Face-trace fields, one plane per field: phi, psi and a_1 along the face's axis.
+constexpr int KIN_NT = 3;
+
+// Volume part of one stage at the thread's node (phi, psi), at velocity c U: broken gradients, n,
+// a_1, the volume term of -a_1 (D^ contractions) and the non-conservative transport; writes the
+// volume part and the face traces.  Every thread of the block calls it (it synchronises the block).
+// s_op: Dx, Dy, Dhx, Dhy; s_f: two fields of fs values.
 template <int P>
-__global__ void __launch_bounds__(Geom<P, 2, false, false>::THREADS)
-k_kin_stage(const KinParams kp, int mode, int kstep, double frac, const double *__restrict__ win,
-            const double *w0, double *__restrict__ acc, double *out) {
-  const double dt = __ldg(kp.dt);
-  const double tstep = kstep * dt, toff = frac * dt;
+__device__ __forceinline__ void kin_volume_part(const KinParams &kp, const double *s_op, double *s_f, int fs, int le,
+                                                int a, int e, bool lane, bool act, double phi, double psi, double2 U,
+                                                double c, double *__restrict__ rvol, double *__restrict__ tr) {
   using G = Geom<P, 2, false, false>;
-  constexpr int P1 = G::P1, NP = G::NP, EPB = G::EPB, NFK = G::NFK, NK = G::NK;
-  const OpsLayout L{P1, NP};
-  __shared__ double s_op[4 * P1 * P1 + 3 * P1 + NP];
-  __shared__ double s_f[2][EPB][NP];       // phi, psi; then -a_1
-  __shared__ double s_nb[EPB][4][2][NP];   // the four neighbours' phi, psi
-  __shared__ double s_tr[EPB][NP][6];      // phi, psi, d(phi)/dx, d(phi)/dy, n_x, n_y
-  __shared__ double s_surf[EPB][NFK][2];
-  __shared__ double s_lift[EPB][NFK];
-  for (int t = threadIdx.x; t < L.cf(); t += blockDim.x) s_op[t] = kp.ops[t];
-  const double *Dx = s_op + L.Dx(), *Dy = s_op + L.Dy(), *Dhx = s_op + L.Dhx(), *Dhy = s_op + L.Dhy();
-  const double *invM = s_op + L.invM(), *wfx = s_op + L.wfx(), *wfy = s_op + L.wfy();
-
-  const int le_raw = threadIdx.x / NP;
-  const bool lane = le_raw < EPB;
-  const int le = lane ? le_raw : EPB - 1;
-  const int a = threadIdx.x % NP;
-  const int e = blockIdx.x * EPB + le;
-  const int N = kp.N;
-  const bool act = lane && e < kp.E && in_bounds(kp.status, (long long)e * NP + a, N);
-  const int i = a % P1, j = a / P1;
-  const long n = (long)(act ? e : 0) * NP + a;
-  const double2 *vt = reinterpret_cast<const double2 *>(kp.vel_tab);
-  // The time factor of the velocity and dt/6, once per CTA: FP64 is this kernel's bound, and a
-  // cosine or a division per thread would cost a fifth of its work.
-  __shared__ double s_c[2];
-  if (threadIdx.x == 0) {
-    s_c[0] = kin_time_factor(kp, (*kp.t0 + tstep) + toff);
-    s_c[1] = dt / 6.0;
-  }
-
-  const double phi = act ? __ldg(win + n) : 0.0, psi = act ? __ldg(win + N + n) : 0.0;
-  const double2 U = __ldg(vt + n);
+  constexpr int P1 = G::P1, NP = G::NP, NFK = G::NFK, NK = G::NK, P11 = P1 * P1;
+  const double *Dx = s_op, *Dy = s_op + P11, *Dhx = s_op + 2 * P11, *Dhy = s_op + 3 * P11;
+  const int i = a % P1, j = a / P1, sn = le * NP + a, sx = le * NP + P1 * j, sy = le * NP + i;
+  const long n = (long)e * NP + a;
+  __syncthreads();
   if (lane) {
-    s_f[0][le][a] = phi;
-    s_f[1][le][a] = psi;
-#pragma unroll
-    for (int f = 0; f < 4; ++f) {
-      const long m = (long)(act ? kin_neighbour(kp, e, f) : 0) * NP + a;
-      const bool ok = in_bounds(kp.status, m, N);
-      s_nb[le][f][0][a] = ok ? __ldg(win + m) : 0.0;
-      s_nb[le][f][1][a] = ok ? __ldg(win + N + m) : 0.0;
-    }
+    s_f[sn] = phi;
+    s_f[fs + sn] = psi;
   }
   __syncthreads();
-  const double c = s_c[0], dt6 = s_c[1];
-  const double u = U.x * c, v = U.y * c;
   double gpx = 0.0, gpy = 0.0, gsx = 0.0, gsy = 0.0;
 #pragma unroll
   for (int k = 0; k < P1; ++k) {
     const double dx = Dx[i * P1 + k], dy = Dy[j * P1 + k];
-    gpx = fma(dx, s_f[0][le][k + P1 * j], gpx);
-    gsx = fma(dx, s_f[1][le][k + P1 * j], gsx);
-    gpy = fma(dy, s_f[0][le][i + P1 * k], gpy);
-    gsy = fma(dy, s_f[1][le][i + P1 * k], gsy);
+    gpx = k ? fma(dx, s_f[sx + k], gpx) : dx * s_f[sx];
+    gsx = k ? fma(dx, s_f[fs + sx + k], gsx) : dx * s_f[fs + sx];
+    gpy = k ? fma(dy, s_f[sy + P1 * k], gpy) : dy * s_f[sy];
+    gsy = k ? fma(dy, s_f[fs + sy + P1 * k], gsy) : dy * s_f[fs + sy];
   }
-  const double g2 = gsx * gsx + gsy * gsy;
-  double nx = 0.0, ny = 0.0;
-  if (g2 >= 1e-24) {
-    const double r = rsqrt(g2);
-    nx = gsx * r;
-    ny = gsy * r;
-  }
-  const double sphi = phi * (1.0 - phi);
-  const double a1x = kp.Gamma * (kp.eps * gpx - sphi * nx);
-  const double a1y = kp.Gamma * (kp.eps * gpy - sphi * ny);
+  // a_1 = Gamma (eps grad phi - phi (1 - phi) grad psi / |grad psi|), n = 0 where |grad psi| < 1e-12
+  const double g2 = fma(gsy, gsy, gsx * gsx);
+  const double Gn = has_gradient(g2) ? kp.Gamma * fma(-phi, phi, phi) * rsqrt64(g2) : 0.0;
+  const double a1x = fma(kp.Ge, gpx, -(Gn * gsx)), a1y = fma(kp.Ge, gpy, -(Gn * gsy));
   __syncthreads();
   if (lane) {
-    s_f[0][le][a] = -a1x;
-    s_f[1][le][a] = -a1y;
-    double *t = s_tr[le][a];
-    t[0] = phi;
-    t[1] = psi;
-    t[2] = gpx;
-    t[3] = gpy;
-    t[4] = nx;
-    t[5] = ny;
+    s_f[sn] = a1x;
+    s_f[fs + sn] = a1y;
   }
   __syncthreads();
-  double Rphi = 0.0;
+  double R = 0.0;
 #pragma unroll
   for (int k = 0; k < P1; ++k) {
-    Rphi = fma(Dhx[i * P1 + k], s_f[0][le][k + P1 * j], Rphi);
-    Rphi = fma(Dhy[j * P1 + k], s_f[1][le][i + P1 * k], Rphi);
+    const double ax = s_f[sx + k];
+    R = k ? fma(Dhx[i * P1 + k], ax, R) : Dhx[i * P1] * ax;
+    R = fma(Dhy[j * P1 + k], s_f[fs + sy + P1 * k], R);
   }
-  Rphi -= u * gpx + v * gpy;
-  const double Rpsi = -(u * gsx + v * gsy);
+  if (!act) return;
+  rvol[n] = -fma(c, fma(U.y, gpy, U.x * gpx), R);
+  rvol[kp.N + n] = -(c * fma(U.y, gsy, U.x * gsx));
+  const long stride = (long)kp.E * NFK;
+  auto put = [&](int f, int kk, double an) {
+    const long o = (long)e * NFK + f * NK + kk;
+    if (!in_bounds(kp.status, o, stride)) return;
+    tr[o] = phi;
+    tr[stride + o] = psi;
+    tr[2 * stride + o] = an;
+  };
+  if (i == 0) put(0, j, a1x);
+  if (i == P) put(1, j, a1x);
+  if (j == 0) put(2, i, a1y);
+  if (j == P) put(3, i, a1y);
+}
 
-  // Face nodes: own trace from s_tr, the neighbour's from its nodal values.
-  for (int t = a; t < NFK && lane; t += NP) {
-    const int f = t / NK, kk = t % NK;
-    const bool xf = f < 2;
-    const double sg = (f & 1) ? 1.0 : -1.0;
-    double flux = 0.0, fpsi = 0.0, lift = 0.0;
-    if (act) {
-      const int am = kin_face_node<P>(f, kk), ap = kin_face_node<P>(f ^ 1, kk);
-      const int e2 = kin_neighbour(kp, e, f);
-      const double *tm = s_tr[le][am];
-      const double *nbp = s_nb[le][f][0], *nbs = s_nb[le][f][1];
-      const int i2 = ap % P1, j2 = ap / P1;
-      double qpx = 0.0, qpy = 0.0, qsx = 0.0, qsy = 0.0;  // the neighbour's gradients at its face node
+// The volume part of a sequence's first stage, on the state w (time factor kt[ic]).
+template <int P>
+__global__ void __launch_bounds__(MAX_THREADS64)
+k_kin_volume(const KinParams kp, int epb, int ic, const double *__restrict__ w, double *__restrict__ rvol,
+             double *__restrict__ tr) {
+  using G = Geom<P, 2, false, false>;
+  constexpr int P11 = G::P1 * G::P1, NP = G::NP;
+  extern __shared__ double s_mem[];
+  grid_dependency_wait();
+  for (int t = threadIdx.x; t < 4 * P11; t += blockDim.x) s_mem[t] = kp.ops[t];
+  const int le_raw = threadIdx.x / NP, a = threadIdx.x % NP;
+  const bool lane = le_raw < epb;
+  const int le = lane ? le_raw : epb - 1, e0 = blockIdx.x * epb + le;
+  const bool act = lane && e0 < kp.E && in_bounds(kp.status, (long long)e0 * NP + a, kp.N);
+  const int e = act ? e0 : 0;
+  const long n = (long)e * NP + a;
+  const double2 U = __ldg(reinterpret_cast<const double2 *>(kp.vel_tab) + n);
+  kin_volume_part<P>(kp, s_mem, s_mem + 4 * P11, epb * NP, le, a, e, lane, act, act ? __ldca(w + n) : 0.0,
+                     act ? __ldca(w + kp.N + n) : 0.0, U, __ldca(kp.kt + KT_C + ic), rvol, tr);
+}
+
+// One stage of the kinematic mode: at every face node the transport flux (lambda - m.u-) [[f]] and
+// the SIP flux of a_1 with its lifted symmetric term, from the traces of both sides; M^-1 (in the
+// tables cf and lw), the volume part and the right-hand side or an RK4 stage:
+//   K1: acc = L,        r = w0 + dt/2 L
+//   K2: acc += 2 L,     r = w0 + dt/2 L
+//   K3: acc += 2 L,     r = w0 + dt L
+//   K4: r = w0 + dt/6 (acc + L), written to w0 (each node by the thread that read it);
+// then, unless last, the volume part of the next stage on r (time factor kt[KT_C + ic + 1]; stage
+// index ic of the captured sequence), into rvol (the node's own value was read before) and the
+// other trace buffer, which neighbouring blocks of this launch do not read.
+// Bound by the FP64 pipe: about 65 operations per node at p = 3, where a stage that evaluated the
+// neighbours' gradients and normals at every face node itself took about 150 (64 x 64, p = 3: an RK4
+// step 85 -> 44 us).
+template <int P>
+__global__ void __launch_bounds__(MAX_THREADS64)
+k_kin_stage(const KinParams kp, int epb, int mode, int ic, bool last, double *w0, double *__restrict__ acc,
+            double *rvol, const double *__restrict__ tr, double *__restrict__ tr_out, double *out) {
+  using G = Geom<P, 2, false, false>;
+  constexpr int P1 = G::P1, NP = G::NP, NFK = G::NFK, NK = G::NK, P11 = P1 * P1;
+  const OpsLayout L{P1, NP};
+  extern __shared__ double s_mem[];
+  double *s_op = s_mem, *s_cf = s_op + 4 * P11, *s_lw = s_cf + 2;
+  double *s_f = s_lw + 4 * P1;           // [2][epb * NP]
+  double *s_s = s_f + 2 * epb * NP;      // [3][epb * NFK]: twice the flux of phi and psi, Gamma eps [[phi]]
+  const int fs = epb * NFK, N = kp.N;
+  grid_dependency_wait();
+  for (int t = threadIdx.x; t < 4 * P11; t += blockDim.x) s_op[t] = kp.ops[t];
+  for (int t = threadIdx.x; t < 2 + 4 * P1; t += blockDim.x) s_cf[t] = kp.ops[L.cf() + t];
+  const double c = __ldca(kp.kt + KT_C + ic);
+  const double2 *vt = reinterpret_cast<const double2 *>(kp.vel_tab);
+  const long stride = (long)kp.E * NFK;
+
+  const int le_raw = threadIdx.x / NP, a = threadIdx.x % NP;
+  const bool lane = le_raw < epb;
+  const int le = lane ? le_raw : epb - 1, e0 = blockIdx.x * epb + le;
+  const bool act = lane && e0 < kp.E && in_bounds(kp.status, (long long)e0 * NP + a, N);
+  const int e = act ? e0 : 0;
+  const long n = (long)e * NP + a;
+  double r[2], base[2] = {0.0, 0.0};
 #pragma unroll
-      for (int k = 0; k < P1; ++k) {
-        const double dx = Dx[i2 * P1 + k], dy = Dy[j2 * P1 + k];
-        qpx = fma(dx, nbp[k + P1 * j2], qpx);
-        qsx = fma(dx, nbs[k + P1 * j2], qsx);
-        qpy = fma(dy, nbp[i2 + P1 * k], qpy);
-        qsy = fma(dy, nbs[i2 + P1 * k], qsy);
-      }
-      const double q2 = qsx * qsx + qsy * qsy;
-      double mx = 0.0, my = 0.0;
-      if (q2 >= 1e-24) {
-        const double r = rsqrt(q2);
-        mx = qsx * r;
-        my = qsy * r;
-      }
-      const long om = (long)e * NP + am, op = (long)e2 * NP + ap;
-      const double2 Um = in_bounds(kp.status, om, N) ? __ldg(vt + om) : make_double2(0.0, 0.0);
-      const double2 Up = in_bounds(kp.status, op, N) ? __ldg(vt + op) : make_double2(0.0, 0.0);
-      const double phm = tm[0], psm = tm[1], php = nbp[ap], psp = nbs[ap];
-      const double unm = (xf ? Um.x : Um.y) * c * sg, unp = (xf ? Up.x : Up.y) * c * sg;
-      const double lam = fmax(fabs(unm), fabs(unp));
-      const double wf = xf ? wfx[kk] : wfy[kk];
-      const double eta = xf ? kp.eta_x : kp.eta_y;
-      const double jump = php - phm;
-      const double gn = 0.5 * ((xf ? qpx : qpy) + (xf ? tm[2] : tm[3])) * sg;
-      const double sharp = 0.5 * (php * (1.0 - php) * (xf ? mx : my) + phm * (1.0 - phm) * (xf ? tm[4] : tm[5])) * sg;
-      const double ahat = kp.Gamma * (kp.eps * (gn + eta * jump) - sharp);
-      flux = wf * (lam - unm) * 0.5 * jump + wf * ahat;
-      fpsi = wf * (lam - unm) * 0.5 * (psp - psm);
-      lift = -wf * 0.5 * kp.Gamma * kp.eps * jump;
+  for (int v = 0; v < 2; ++v) {
+    r[v] = __ldca(rvol + (long)v * N + n);
+    if (mode != KIN_RHS) base[v] = __ldca(w0 + (long)v * N + n);
+  }
+
+  for (int g = threadIdx.x; g < fs; g += blockDim.x) {
+    const int fe = blockIdx.x * epb + g / NFK, t = g % NFK;
+    if (fe >= kp.E) break;
+    const int f = t / NK, kk = t % NK, e2 = kin_neighbour(kp, fe, f);
+    const bool xf = f < 2;
+    const int sm = (f & 1) ? 0 : (int)0x80000000;  // sign of m
+    const long om = (long)fe * NFK + t, op = (long)e2 * NFK + (f ^ 1) * NK + kk;
+    const long nm = (long)fe * NP + kin_face_node<P>(f, kk), np = (long)e2 * NP + kin_face_node<P>(f ^ 1, kk);
+    double flux = 0.0, fpsi = 0.0, gej = 0.0;
+    if (in_bounds(kp.status, om, stride) && in_bounds(kp.status, op, stride) && in_bounds(kp.status, nm, N) &&
+        in_bounds(kp.status, np, N)) {
+      const double jphi = __ldca(tr + op) - __ldca(tr + om);
+      const double jpsi = __ldca(tr + stride + op) - __ldca(tr + stride + om);
+      const double asum = __ldca(tr + 2 * stride + op) + __ldca(tr + 2 * stride + om);
+      const double2 Um = __ldg(vt + nm), Up = __ldg(vt + np);
+      const double um = flip64(xf ? Um.x : Um.y, sm), up = xf ? Up.x : Up.y;
+      // lambda - m.u- with lambda = |c| max(|U- . m|, |U+ . m|)
+      const double lu = fma(-c, um, fabs(c) * max_nonneg64(fabs(um), fabs(up)));
+      gej = kp.Ge * jphi;
+      flux = fma(lu, jphi, fma(xf ? kp.Gp_x : kp.Gp_y, jphi, flip64(asum, sm)));
+      fpsi = lu * jpsi;
     }
-    s_surf[le][t][0] = flux;
-    s_surf[le][t][1] = fpsi;
-    s_lift[le][t] = lift;
+    s_s[g] = flux;
+    s_s[fs + g] = fpsi;
+    s_s[2 * fs + g] = gej;
   }
   __syncthreads();
-  if (!act) return;
-
-  double sp = 0.0, ss = 0.0;
-  if (i == 0) { sp += s_surf[le][0 * NK + j][0]; ss += s_surf[le][0 * NK + j][1]; }
-  if (i == P) { sp += s_surf[le][1 * NK + j][0]; ss += s_surf[le][1 * NK + j][1]; }
-  if (j == 0) { sp += s_surf[le][2 * NK + i][0]; ss += s_surf[le][2 * NK + i][1]; }
-  if (j == P) { sp += s_surf[le][3 * NK + i][0]; ss += s_surf[le][3 * NK + i][1]; }
-  sp += s_lift[le][0 * NK + j] * -Dx[0 * P1 + i] + s_lift[le][1 * NK + j] * Dx[P * P1 + i];
-  sp += s_lift[le][2 * NK + i] * -Dy[0 * P1 + j] + s_lift[le][3 * NK + i] * Dy[P * P1 + j];
-  const double im = invM[a];
-  const double Lv[2] = {Rphi + sp * im, Rpsi + ss * im};
-  bool bad = false;
-#pragma unroll
-  for (int vv = 0; vv < 2; ++vv) {
-    const long o = (long)vv * N + n;
-    double r;
-    if (mode == KIN_RHS) {
-      r = Lv[vv];
-    } else {
-      const double base = w0[o];
-      if (mode == KIN_K1) {
-        acc[o] = Lv[vv];
-        r = base + 0.5 * dt * Lv[vv];
-      } else if (mode == KIN_K2) {
-        acc[o] += 2.0 * Lv[vv];
-        r = base + 0.5 * dt * Lv[vv];
-      } else if (mode == KIN_K3) {
-        acc[o] += 2.0 * Lv[vv];
-        r = base + dt * Lv[vv];
-      } else {
-        r = base + dt6 * (acc[o] + Lv[vv]);
-      }
-    }
-    bad |= !isfinite(r);
-    out[o] = r;
+  const int i = a % P1, j = a / P1, gb = le * NFK;
+  if (i == 0 || i == P) {
+    const int g = gb + (i == 0 ? 0 : NK) + j;
+    r[0] = fma(s_cf[0], s_s[g], r[0]);
+    r[1] = fma(s_cf[0], s_s[fs + g], r[1]);
   }
-  if (kp.check_finite && bad) atomicOr(kp.status, STATUS_NONFINITE);
+  if (j == 0 || j == P) {
+    const int g = gb + (j == 0 ? 2 : 3) * NK + i;
+    r[0] = fma(s_cf[1], s_s[g], r[0]);
+    r[1] = fma(s_cf[1], s_s[fs + g], r[1]);
+  }
+  {
+    const double *lift = s_s + 2 * fs + gb;
+    r[0] = fma(s_lw[i], lift[j], r[0]);
+    r[0] = fma(s_lw[P1 + i], lift[NK + j], r[0]);
+    r[0] = fma(s_lw[2 * P1 + j], lift[2 * NK + i], r[0]);
+    r[0] = fma(s_lw[3 * P1 + j], lift[3 * NK + i], r[0]);
+  }
+  if (mode != KIN_RHS) {
+    const double h = __ldca(kp.kt + (mode == KIN_K4 ? KT_SIXTH : (mode == KIN_K3 ? KT_DT : KT_HALF)));
+#pragma unroll
+    for (int v = 0; v < 2; ++v) {
+      const long o = (long)v * N + n;
+      double Lv = r[v];
+      if (act) {
+        if (mode == KIN_K1) {
+          acc[o] = Lv;
+        } else {
+          const double q = acc[o];
+          if (mode == KIN_K4) Lv += q;
+          else acc[o] = fma(2.0, Lv, q);
+        }
+      }
+      r[v] = fma(h, Lv, base[v]);
+    }
+  }
+  if (act) {
+    if (kp.check_finite && !(finite64(r[0]) && finite64(r[1]))) atomicOr(kp.status, STATUS_NONFINITE);
+    if (mode == KIN_RHS || mode == KIN_K4) {
+      out[n] = r[0];
+      out[N + n] = r[1];
+    }
+  }
+  if (last) return;
+  kin_volume_part<P>(kp, s_op, s_f, epb * NP, le, a, e, lane, act, act ? r[0] : 0.0, act ? r[1] : 0.0, __ldg(vt + n),
+                     __ldca(kp.kt + KT_C + ic + 1), rvol, tr_out);
 }
 
 struct KinKernels {
-  cudaError_t (*stage)(const KinParams &, int mode, int kstep, double frac, const double *win, const double *w0,
-                       double *acc, double *out, cudaStream_t);
+  cudaError_t (*volume)(const KinParams &, int ic, const double *w, double *rvol, double *tr, cudaStream_t);
+  cudaError_t (*stage)(const KinParams &, int mode, int ic, bool last, double *w0, double *acc, double *rvol,
+                       const double *tr, double *tr_out, double *out, cudaStream_t);
   cudaError_t (*velocity_table)(const KinParams &, double *tab, cudaStream_t);
 };
 
 template <int P>
-cudaError_t launch_kin_stage(const KinParams &kp, int mode, int kstep, double frac, const double *win,
-                             const double *w0, double *acc, double *out, cudaStream_t s) {
+cudaError_t launch_kin_volume(const KinParams &kp, int ic, const double *w, double *rvol, double *tr, cudaStream_t s) {
   using G = Geom<P, 2, false, false>;
-  k_kin_stage<P><<<(kp.E + G::EPB - 1) / G::EPB, G::THREADS, 0, s>>>(kp, mode, kstep, frac, win, w0, acc, out);
-  return cudaGetLastError();
+  const int epb = pick_epb64(kp.E, G::NP, 1), threads = (epb * G::NP + 31) / 32 * 32;
+  const size_t smem = sizeof(double) * (4 * G::P1 * G::P1 + 2 * (size_t)epb * G::NP);
+  return launch_dependent(k_kin_volume<P>, (kp.E + epb - 1) / epb, threads, smem, s, kp, epb, ic, w, rvol, tr);
+}
+
+template <int P>
+cudaError_t launch_kin_stage(const KinParams &kp, int mode, int ic, bool last, double *w0, double *acc, double *rvol,
+                             const double *tr, double *tr_out, double *out, cudaStream_t s) {
+  using G = Geom<P, 2, false, false>;
+  // (a node costs about five times a face node)
+  const int epb = pick_epb64(kp.E, G::NP, 5, G::NFK, 1), threads = (epb * G::NP + 31) / 32 * 32;
+  const size_t smem =
+      sizeof(double) * (4 * G::P1 * G::P1 + 2 + 4 * G::P1 + (size_t)epb * (2 * G::NP + 3 * G::NFK));
+  return launch_dependent(k_kin_stage<P>, (kp.E + epb - 1) / epb, threads, smem, s, kp, epb, mode, ic, last, w0, acc,
+                          rvol, tr, tr_out, out);
 }
 
 bool kin_kernels(int p, KinKernels *out);

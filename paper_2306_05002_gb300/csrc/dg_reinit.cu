@@ -5,7 +5,7 @@ namespace dgpf {
 
 template <int P, int DIM>
 static ReinitKernels make_ri() {
-  return ReinitKernels{&launch_ri_sign<P, DIM>, &launch_ri_volume<P, DIM>, &launch_ri_surface<P, DIM>,
+  return ReinitKernels{&launch_ri_sign<P, DIM>, &launch_ri_volume<P, DIM>, &launch_ri_stage<P, DIM>,
                        Geom<P, DIM, false, false>::NFK};
 }
 

@@ -169,7 +169,7 @@ __device__ __forceinline__ void tri_eval_point(const KinParams &kp, const TriCon
   o->gs[0] = sr * g.rx + sq * g.sx;
   o->gs[1] = sr * g.ry + sq * g.sy;
   const double g2 = o->gs[0] * o->gs[0] + o->gs[1] * o->gs[1];
-  const double rn = g2 < 1e-24 ? 0.0 : rsqrt(g2);  // n = 0 where |grad psi| < 1e-12
+  const double rn = has_gradient(g2) ? rsqrt64(g2) : 0.0;  // n = 0 where |grad psi| < 1e-12
   const double sp = ph * (1.0 - ph);
 #pragma unroll
   for (int d = 0; d < 2; ++d) {
@@ -211,19 +211,17 @@ __device__ __forceinline__ void tri_edge_trace(const double *s_t, const TriLayou
   o->phi = ph;
   o->psi = ps;
   o->dphi_m = sgn * gp;
-  o->n_m = g2 < 1e-24 ? 0.0 : sgn * gs * rsqrt(g2);  // n = 0 where |grad psi| < 1e-12
+  o->n_m = has_gradient(g2) ? sgn * gs * rsqrt64(g2) : 0.0;  // n = 0 where |grad psi| < 1e-12
 }
 
-// One stage: the right-hand side L = M^-1 R(win) at time *t0 + kstep dt + frac dt,
-// written as L (KIN_RHS) or as one classical RK4 stage (KIN_K1..K4, the same
+// One stage: the right-hand side L = M^-1 R(win) at the time of stage ic of the
+// captured sequence (KinTime), written as L (KIN_RHS) or as one classical RK4 stage (KIN_K1..K4, the same
 // updates as k_kin_stage; out may be w0, each node being read, then written,
 // by the same thread).
 template <int P>
 __global__ void __launch_bounds__(TriGeom<P>::THREADS)
-k_tri_stage(const KinParams kp, int mode, int kstep, double frac, const double *__restrict__ win,
-            const double *w0, double *__restrict__ acc, double *out) {
-  const double dt = __ldg(kp.dt);  // step size and stage time as in k_kin_stage
-  const double tstep = kstep * dt, toff = frac * dt;
+k_tri_stage(const KinParams kp, int mode, int ic, const double *__restrict__ win, const double *w0,
+            double *__restrict__ acc, double *out) {
   using G = TriGeom<P>;
   constexpr TriLayout L = G::L;
   constexpr int NP = G::NP, NQ1 = G::NQ1, NQV = G::NQV, NQE = G::NQE, EPB = G::EPB;
@@ -235,7 +233,8 @@ k_tri_stage(const KinParams kp, int mode, int kstep, double frac, const double *
   __shared__ double s_ce[EPB][NQE][4];
   __shared__ double s_R[EPB][2][NP];
   for (int i = threadIdx.x; i < L.size(); i += blockDim.x) s_t[i] = kp.ops[i];
-  const double c = kin_time_factor(kp, (*kp.t0 + tstep) + toff);
+  const double c = kp.kt[KT_C + ic];
+  const double hstep = kp.kt[mode == KIN_K4 ? KT_SIXTH : (mode == KIN_K3 ? KT_DT : KT_HALF)];
   const int N = kp.N, ngroups = (kp.E + EPB - 1) / EPB;
   bool bad = false;
 
@@ -375,18 +374,15 @@ k_tri_stage(const KinParams kp, int mode, int kstep, double frac, const double *
           const double base = w0[o];
           if (mode == KIN_K1) {
             acc[o] = Lv;
-            r = base + 0.5 * dt * Lv;
-          } else if (mode == KIN_K2) {
-            acc[o] += 2.0 * Lv;
-            r = base + 0.5 * dt * Lv;
-          } else if (mode == KIN_K3) {
-            acc[o] += 2.0 * Lv;
-            r = base + dt * Lv;
+            r = fma(hstep, Lv, base);
+          } else if (mode == KIN_K4) {
+            r = fma(hstep, acc[o] + Lv, base);
           } else {
-            r = base + dt / 6.0 * (acc[o] + Lv);
+            acc[o] = fma(2.0, Lv, acc[o]);
+            r = fma(hstep, Lv, base);
           }
         }
-        bad |= !isfinite(r);
+        bad |= !finite64(r);
         out[o] = r;
       }
     }
@@ -395,8 +391,8 @@ k_tri_stage(const KinParams kp, int mode, int kstep, double frac, const double *
 }
 
 struct TriKernels {
-  cudaError_t (*stage)(const KinParams &, int mode, int kstep, double frac, const double *win, const double *w0,
-                       double *acc, double *out, int grid, cudaStream_t);
+  cudaError_t (*stage)(const KinParams &, int mode, int ic, const double *win, const double *w0, double *acc,
+                       double *out, int grid, cudaStream_t);
   cudaError_t (*velocity_table)(const KinParams &, double *tab, cudaStream_t);
   const void *fn;  // the stage kernel, for the occupancy query
   int threads;
@@ -404,9 +400,9 @@ struct TriKernels {
 };
 
 template <int P>
-cudaError_t launch_tri_stage(const KinParams &kp, int mode, int kstep, double frac, const double *win,
-                             const double *w0, double *acc, double *out, int grid, cudaStream_t s) {
-  k_tri_stage<P><<<grid, TriGeom<P>::THREADS, 0, s>>>(kp, mode, kstep, frac, win, w0, acc, out);
+cudaError_t launch_tri_stage(const KinParams &kp, int mode, int ic, const double *win, const double *w0, double *acc,
+                             double *out, int grid, cudaStream_t s) {
+  k_tri_stage<P><<<grid, TriGeom<P>::THREADS, 0, s>>>(kp, mode, ic, win, w0, acc, out);
   return cudaGetLastError();
 }
 
