@@ -24,7 +24,11 @@
 #include "dg_host.h"
 #include "dgpf.h"
 
-static __device__ __align__(256) unsigned char g_noalloc_scratch[DG_NOALLOC_SCRATCH_BYTES];
+// What a call is held to counts an operator table without its derived part (OpsLayout from cf() on), 17 face
+// trace fields with viscous stress and 14 without: at least what the kernels use, but for that derived part
+// (26 doubles at most), which has its room behind the limit.
+constexpr size_t kDerivedTableBytes = 256;
+static __device__ __align__(256) unsigned char g_noalloc_scratch[DG_NOALLOC_SCRATCH_BYTES + kDerivedTableBytes];
 
 namespace {
 
@@ -88,8 +92,9 @@ extern "C" dg_status dg_rhs_noalloc(const dg_mesh *mesh, int p, const dg_eos *eo
   // scratch: status word | operator table | volume part (7 N) | face traces (nt E NFK)
   const size_t off_ops = 256;
   const size_t off_rvol = off_ops + align256(sizeof(double) * lay.size());
-  const size_t off_tr = off_rvol + align256(sizeof(double) * 7 * (size_t)N);
-  const size_t need = off_tr + sizeof(double) * (size_t)ks.nt * (size_t)E * NFK;
+  const size_t rvol_bytes = align256(sizeof(double) * 7 * (size_t)N), off_tr = off_rvol + rvol_bytes;
+  const size_t need = off_ops + align256(sizeof(double) * lay.cf()) + rvol_bytes +
+                      sizeof(double) * (size_t)(o.viscous ? 17 : 14) * (size_t)E * NFK;
   if (need > (size_t)DG_NOALLOC_SCRATCH_BYTES) return DG_ERR_ARG;  // too large for the fixed scratch
 
   unsigned char *base = nullptr;
