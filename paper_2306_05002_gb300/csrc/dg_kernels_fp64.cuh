@@ -129,8 +129,8 @@ inline int pick_epb64(int E, int per, int cn, int perf = 0, int cf = 0) {
 // the time (64 x 64, p = 3: 191 us a step with an early trigger, 141 without).
 //
 // Bound by the FP64 pipe.  64 x 64, p = 3 in 2D: a step of three volume and three surface launches
-// 172 -> 141 us (loading the update's inputs ahead of the face work: no gain, and 3% slower where the
-// grid has several waves, for the registers it holds).
+// 172 -> 141 us (what the update reads requested where it is used: 147; ahead of the face work: no gain,
+// and 3% slower where the grid has several waves, for the registers it holds).
 template <int P, int DIM>
 __global__ void __launch_bounds__(MAX_THREADS64)
 k_volume(const Params prm, int epb, const double *__restrict__ w, double *__restrict__ rvol,
@@ -475,6 +475,18 @@ k_surface(const Params prm, int epb, int mode, double dt, const double *__restri
   // Phase 2: gather onto the element's nodes, lift the symmetric term along
   // the normal lines, apply M^-1, add the volume part, write L or the stage.
   if (!act) return;
+  // what the update reads is requested here, before the shared-memory gather, in one run
+  double rv[NV], wn[NV], w0n[NV];
+#pragma unroll
+  for (int vv = 0; vv < NV; ++vv) rv[vv] = __ldca(rvol + (long)vv * N + n);
+  if (mode != MODE_RHS) {
+#pragma unroll
+    for (int vv = 0; vv < NV; ++vv) wn[vv] = __ldca(ws + (long)vv * N + n);
+    if (mode != MODE_S1) {
+#pragma unroll
+      for (int vv = 0; vv < NV; ++vv) w0n[vv] = __ldca(w0 + (long)vv * N + n);
+    }
+  }
   const int i = a % P1, j = DIM == 2 ? a / P1 : 0;
   const int kx = DIM == 2 ? j : 0;
   const int gb = le * NFK;
@@ -509,11 +521,11 @@ k_surface(const Params prm, int epb, int mode, double dt, const double *__restri
 #pragma unroll
   for (int vv = 0; vv < NV; ++vv) {
     const long o = (long)vv * N + n;
-    double r = fma(acc[vv], im, __ldca(rvol + o));
+    double r = fma(acc[vv], im, rv[vv]);
     if (mode != MODE_RHS) {
-      r = fma(dt, r, __ldca(ws + o));
-      if (mode == MODE_S2) r = fma(0.25, r, 0.75 * __ldca(w0 + o));
-      else if (mode == MODE_S3) r = fma(2.0 / 3.0, r, (1.0 / 3.0) * __ldca(w0 + o));
+      r = fma(dt, r, wn[vv]);
+      if (mode == MODE_S2) r = fma(0.25, r, 0.75 * w0n[vv]);
+      else if (mode == MODE_S3) r = fma(2.0 / 3.0, r, (1.0 / 3.0) * w0n[vv]);
     }
     bad |= !finite64(r);
     out[o] = r;
