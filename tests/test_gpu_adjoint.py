@@ -316,3 +316,25 @@ def test_adjoint_rejects_pressure_boundary(dg):
         s.dg_rhs_vjp(w, w.clone())
     s.close()
 
+
+
+@pytest.mark.parametrize("bc", [("noslip", "slip", "periodic", "periodic"), ("periodic", "periodic", "slip", "noslip"),
+                                ("slip", "noslip", "noslip", "slip")])
+def test_vjp_with_walls_dot_product(dg, bc):
+    """<lam, J v> = <J^T lam, v> on a 5 x 3 mesh with walls: a face is evaluated by the element that has
+    it as its west or south face, east and north faces by their own element only where the mesh ends."""
+    import torch
+    wl = W.drop_2d(n=5, p=3, seed=2)
+    wl.ny, wl.bc = 3, bc
+    wl.w = wl.w[:, : wl.N].copy()
+    w = torch.from_numpy(_broken(wl)).cuda()
+    g = torch.Generator(device="cpu").manual_seed(0)
+    vdir = torch.randn(w.shape, generator=g, dtype=torch.float64).cuda() * w.abs().amax(dim=1, keepdim=True)
+    s = dg.Solver(wl)
+    Lmax = s.dg_rhs(w).abs().amax(dim=1, keepdim=True)
+    lam = torch.randn(w.shape, generator=g, dtype=torch.float64).cuda() / torch.where(Lmax > 0, Lmax, 1.0)
+    h = 1e-9
+    Jv = (s.dg_rhs(w + h * vdir) - s.dg_rhs(w - h * vdir)) / (2 * h)
+    lhs, rhs = float((lam * Jv).sum()), float((s.dg_rhs_vjp(w, lam) * vdir).sum())
+    s.close()
+    assert abs(lhs - rhs) <= 2e-6 * max(abs(lhs), abs(rhs)), (lhs, rhs)
