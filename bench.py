@@ -160,8 +160,11 @@ GATE_CYCLES = 40_000_000
 # --------------------------------------------------------------------------- roofline helpers
 
 KERNEL_SOURCES = {"fp64": ["paper_2306_05002_gb300/csrc/dg_kernels_fp64.cuh",
+                           "paper_2306_05002_gb300/csrc/dg_kernels_full64.cuh",
+                           "paper_2306_05002_gb300/csrc/dg_math64.cuh",
                            "paper_2306_05002_gb300/csrc/dg_common.cuh"],
                   "fp32bulk": ["paper_2306_05002_gb300/csrc/dg_kernels_fp32.cuh",
+                               "paper_2306_05002_gb300/csrc/dg_lines32.cuh",
                                "paper_2306_05002_gb300/csrc/dg_kernels_fp64.cuh",
                                "paper_2306_05002_gb300/csrc/dg_common.cuh",
                                "paper_2306_05002_gb300/csrc/dg_pdl.cuh"]}

@@ -19,6 +19,7 @@
 #include "dg_common.cuh"
 #include "dg_kernels_fp64.cuh"
 #include "dg_kernels_fp32.cuh"
+#include "dg_lines32.cuh"
 #include "dg_batch.cuh"
 #include "dg_adjoint.cuh"
 #include "dg_kin.cuh"
@@ -39,6 +40,23 @@ bool kernels_fp32_p2(int, bool, bool, KernelSet32 *);
 bool kernels_fp32_p3(int, bool, bool, KernelSet32 *);
 bool kernels_fp32_p4(int, bool, bool, KernelSet32 *);
 bool kernels_fp32_p5(int, bool, bool, KernelSet32 *);
+
+KernelSet32 lines_fp32_p1(bool, bool);
+KernelSet32 lines_fp32_p2(bool, bool);
+KernelSet32 lines_fp32_p3(bool, bool);
+KernelSet32 lines_fp32_p4(bool, bool);
+KernelSet32 lines_fp32_p5(bool, bool);
+
+bool lines_fp32(int p, bool viscous, bool st, KernelSet32 *out) {
+  switch (p) {
+    case 1: *out = lines_fp32_p1(viscous, st); return true;
+    case 2: *out = lines_fp32_p2(viscous, st); return true;
+    case 3: *out = lines_fp32_p3(viscous, st); return true;
+    case 4: *out = lines_fp32_p4(viscous, st); return true;
+    case 5: *out = lines_fp32_p5(viscous, st); return true;
+    default: return false;
+  }
+}
 
 void batch_variants_p1(BatchVariant *);
 void batch_variants_p2(BatchVariant *);
@@ -231,6 +249,8 @@ struct dg_ctx {
   KernelSet ks;
   KernelSet32 ks32;
   ParamsF pf;
+  LineParams lp{};      // FP32-bulk, 2D: the line kernels' parameters
+  bool lines = false;   // FP32-bulk: this context runs the line kernels (use_lines32)
   int prec = DG_FP64;
   AdjKernels adj{};
   bool has_adj = false;
@@ -240,6 +260,7 @@ struct dg_ctx {
   float *d_opsf = nullptr, *d_rvol32 = nullptr,
         *d_trace32 = nullptr, *d_rvol32b = nullptr, *d_trace32b = nullptr;
   double *d_ops = nullptr, *d_w1 = nullptr, *d_w2 = nullptr, *d_rvol = nullptr, *d_trace = nullptr;
+  size_t n32 = 0;  // floats of an FP32 node array
   double *d_hstate = nullptr;  // device copy of a host state (dg_step_host), allocated on first use
   double *d_copy64 = nullptr;  // FP32-bulk single steps on a page-locked host state (enqueue_steps32)
   // kinematic mode (dg_kin_create); tri: triangles (one fused kernel per stage)
@@ -436,8 +457,14 @@ extern "C" dg_status dg_create(const dg_mesh *mesh, int p, const dg_eos *eos, do
     return e == cudaSuccess;
   };
   if (!f64) {
-    const size_t n32 = (size_t)SW32 * c->N;  // one padded record per node (inviscid kernels)
-    const size_t t32 = (size_t)TRW32 * c->E * c->NFK;  // one padded record per face node
+    KernelSet32 kl;
+    c->lines = c->dim == 2 && lines_fp32(p, o.viscous != 0, o.surface_tension != 0, &kl) &&
+               use_lines32(P1, o.viscous || o.surface_tension, c->E, kl.wave_tiles);
+    if (c->lines) c->ks32 = kl;
+    // one padded record per node (inviscid kernels) and per face node, or the line kernels' tiles
+    const size_t n32 = c->lines ? line_node_floats(P1, c->E) : (size_t)SW32 * c->N;
+    const size_t t32 = c->lines ? line_trace_floats(P1, c->E) : (size_t)TRW32 * c->E * c->NFK;
+    c->n32 = n32;
     alloc32(&c->d_opsf, opsf.size()) && alloc32(&c->d_hi32[0], n32) && alloc32(&c->d_hi32[1], n32) &&
         alloc32(&c->d_lo32[0], n32) && alloc32(&c->d_lo32[1], n32) && alloc32(&c->d_dd32[0], n32) &&
         alloc32(&c->d_dd32[1], n32) && alloc32(&c->d_rvol32, n32) && alloc32(&c->d_trace32, t32) &&
@@ -470,6 +497,7 @@ extern "C" dg_status dg_create(const dg_mesh *mesh, int p, const dg_eos *eos, do
   }
   q.ops = c->d_ops;
   q.status = c->d_status;
+  if (c->lines) c->lp = line_params(c->prm, P1, opsf.data(), c->d_opsf);
   *out = c;
   return DG_OK;
 }
@@ -561,11 +589,11 @@ static dg_status run_stage(dg_ctx *c, int mode, double dt, const double *w0, con
 // the state into the internal hi part (the lo part is not needed) and the
 // surface kernel writes L in FP64.
 static dg_status rhs32(dg_ctx *c, const double *w64, double *L, cudaStream_t s) {
-  cudaError_t e = c->ks32.volume(c->prm, c->pf, c->d_opsf, nullptr, c->d_rvol32, c->d_trace32, w64, c->d_hi32[0],
+  cudaError_t e = c->ks32.volume(c->prm, c->pf, c->lp, c->d_opsf, nullptr, c->d_rvol32, c->d_trace32, w64, c->d_hi32[0],
                                  nullptr, nullptr, s);
   if (e != cudaSuccess) return cuda_fail(c, e, "volume kernel launch");
   const StageIO io{nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, L, nullptr};
-  e = c->ks32.surface(c->prm, c->pf, c->d_opsf, MODE_RHS, 0.f, io, c->d_rvol32, c->d_trace32, s);
+  e = c->ks32.surface(c->prm, c->pf, c->lp, c->d_opsf, MODE_RHS, 0.f, io, c->d_rvol32, c->d_trace32, s);
   if (e != cudaSuccess) return cuda_fail(c, e, "surface kernel launch");
   return DG_OK;
 }
@@ -615,7 +643,7 @@ static dg_status enqueue_steps32(dg_ctx *c, double *w, float dt, int steps, cuda
   int t = 0, a = 0;
   if (steps != 1) copy64 = nullptr;
   // a single step adds its last increment to the FP64 state itself: no lo part is needed
-  cudaError_t e = c->ks32.volume(c->prm, c->pf, c->d_opsf, nullptr, rv[t], tr[t], w, H[a], steps > 1 ? Lo[a] : nullptr,
+  cudaError_t e = c->ks32.volume(c->prm, c->pf, c->lp, c->d_opsf, nullptr, rv[t], tr[t], w, H[a], steps > 1 ? Lo[a] : nullptr,
                                  copy64, s);
   if (e != cudaSuccess) return cuda_fail(c, e, "volume kernel launch");
   for (int k = 0; k < steps; ++k) {
@@ -628,11 +656,11 @@ static dg_status enqueue_steps32(dg_ctx *c, double *w, float dt, int steps, cuda
     const int mode[3] = {MODE_S1, MODE_S2, MODE_S3};
     for (int st = 0; st < 3; ++st) {
       if (st == 2 && last) {
-        e = c->ks32.surface(c->prm, c->pf, c->d_opsf, MODE_S3, dt, io[2], rv[t], tr[t], s);
+        e = c->ks32.surface(c->prm, c->pf, c->lp, c->d_opsf, MODE_S3, dt, io[2], rv[t], tr[t], s);
         if (e != cudaSuccess) return cuda_fail(c, e, "surface kernel launch");
         break;
       }
-      e = c->ks32.surfvol(c->prm, c->pf, c->d_opsf, mode[st], dt, io[st], rv[t], tr[t], rv[t ^ 1], tr[t ^ 1], s);
+      e = c->ks32.surfvol(c->prm, c->pf, c->lp, c->d_opsf, mode[st], dt, io[st], rv[t], tr[t], rv[t ^ 1], tr[t ^ 1], s);
       if (e != cudaSuccess) return cuda_fail(c, e, "fused stage kernel launch");
       t ^= 1;
     }
@@ -821,27 +849,27 @@ extern "C" int dg_time_kernels(dg_ctx *c, const double *w, int nrep, double *ms_
       if (k == 0) c->ks.volume(c->prm, w, c->d_rvol, c->d_trace, s);
       else c->ks.surface(c->prm, MODE_RHS, 0.0, w, w, c->d_rvol, c->d_trace, c->d_w1, s);
     } else if (k == 0) {  // the kernels of a step as dg_step launches them (FP32 state in, FP32 stage out)
-      c->ks32.volume(c->prm, c->pf, c->d_opsf, c->d_hi32[0], c->d_rvol32, c->d_trace32, nullptr, nullptr, nullptr,
+      c->ks32.volume(c->prm, c->pf, c->lp, c->d_opsf, c->d_hi32[0], c->d_rvol32, c->d_trace32, nullptr, nullptr, nullptr,
                      nullptr, s);
     } else if (k == 1) {
       const StageIO io{c->d_hi32[0], nullptr, c->d_dd32[0], c->d_dd32[1], nullptr, nullptr, nullptr, nullptr};
-      c->ks32.surface(c->prm, c->pf, c->d_opsf, MODE_S2, 1e-9f, io, c->d_rvol32, c->d_trace32, s);
+      c->ks32.surface(c->prm, c->pf, c->lp, c->d_opsf, MODE_S2, 1e-9f, io, c->d_rvol32, c->d_trace32, s);
     } else if (k == 2) {
       const StageIO io{c->d_hi32[0], nullptr, c->d_dd32[0], c->d_dd32[1], nullptr, nullptr, nullptr, nullptr};
-      c->ks32.surfvol(c->prm, c->pf, c->d_opsf, MODE_S2, 1e-9f, io, c->d_rvol32, c->d_trace32, c->d_rvol32b,
+      c->ks32.surfvol(c->prm, c->pf, c->lp, c->d_opsf, MODE_S2, 1e-9f, io, c->d_rvol32, c->d_trace32, c->d_rvol32b,
                       c->d_trace32b, s);
     } else if (k == 3) {  // the first stage of a single-step call: reads the FP64 state (hi part only)
-      c->ks32.volume(c->prm, c->pf, c->d_opsf, nullptr, c->d_rvol32b, c->d_trace32b, w, c->d_hi32[1], nullptr,
+      c->ks32.volume(c->prm, c->pf, c->lp, c->d_opsf, nullptr, c->d_rvol32b, c->d_trace32b, w, c->d_hi32[1], nullptr,
                      nullptr, s);
     } else {  // the last stage of a single-step call: adds the last increment to the FP64 state
       const StageIO io{nullptr, nullptr, c->d_dd32[0], nullptr, nullptr, nullptr, tmp64, w};
-      c->ks32.surface(c->prm, c->pf, c->d_opsf, MODE_S3, 1e-9f, io, c->d_rvol32, c->d_trace32, s);
+      c->ks32.surface(c->prm, c->pf, c->lp, c->d_opsf, MODE_S3, 1e-9f, io, c->d_rvol32, c->d_trace32, s);
     }
   };
   if (!f64) {  // the internal state of w (hi, lo) and a zero increment to time the stage kernels on
-    c->ks32.volume(c->prm, c->pf, c->d_opsf, nullptr, c->d_rvol32, c->d_trace32, w, c->d_hi32[0], c->d_lo32[0],
+    c->ks32.volume(c->prm, c->pf, c->lp, c->d_opsf, nullptr, c->d_rvol32, c->d_trace32, w, c->d_hi32[0], c->d_lo32[0],
                    nullptr, s);
-    cudaMemsetAsync(c->d_dd32[0], 0, (size_t)SW32 * c->N * sizeof(float), s);
+    cudaMemsetAsync(c->d_dd32[0], 0, c->n32 * sizeof(float), s);
   }
   cudaEvent_t ev[2];
   for (auto &x : ev) cudaEventCreate(&x);
@@ -887,10 +915,10 @@ extern "C" int dg_kernel_costs(const dg_ctx *c, double *flops, double *bytes, in
   // the volume part, the stage input and the step start (FP32-bulk: the step
   // start and the previous increment), and writes the stage (FP32-bulk: its
   // increment).  FP32-bulk stores traces as padded 12-word records and, in the
-  // inviscid kernels, the state and volume parts as padded 8-word node records.
+  // one-node-per-thread inviscid kernels, the state and volume parts as padded 8-word node records.
   const bool f64 = c->prec == DG_FP64;
   const double nt = f64 ? c->ks.nt : TRW32;
-  const double nw = f64 || visc ? 7 : SW32;
+  const double nw = f64 || visc || c->lines ? 7 : SW32;
   const double word = f64 ? 8.0 : 4.0;
   if (!f64) fv += 3 * 2 * d * P1;  // compression term of the reduced energy
   const double bv = word * (E * Np * (nw + nw) + E * NFK * nt);

@@ -45,6 +45,11 @@
 // hi and lo on load and writing the FP32 internal state), and the last stage
 // can write the FP64 state directly (hi + lo).  With the fused stage kernel
 // (k_surfvol32 below) n steps take 1 + 3n launches.
+//
+// These kernels give a node to a thread: the short chain for 1D problems and for
+// 2D meshes that do not fill the GPU, and the batches (dg_batch.cuh).  Larger
+// 2D meshes run the kernels of dg_lines32.cuh, one element line per thread
+// (use_lines32).
 #pragma once
 
 #include "dg_common.cuh"
@@ -1048,15 +1053,18 @@ k_surfvol32(const Params prm, const ParamsF pf, const float *__restrict__ opsf, 
 // stage on the FP32 state w, or, with w64, on the FP64 state, which it splits
 // into the internal state's hi (w32out) and lo (lo_out, may be NULL) parts and
 // copies into w64copy (may be NULL).
+// Each takes what its own kernels need of Params, ParamsF, LineParams (dg_lines32.cuh) and opsf.
+struct LineParams;
 struct KernelSet32 {
-  cudaError_t (*volume)(const Params &, const ParamsF &, const float *opsf, const float *w, float *rvol,
-                        float *trace, const double *w64, float *w32out, float *lo_out, double *w64copy,
+  cudaError_t (*volume)(const Params &, const ParamsF &, const LineParams &, const float *opsf, const float *w,
+                        float *rvol, float *trace, const double *w64, float *w32out, float *lo_out, double *w64copy,
                         cudaStream_t);
-  cudaError_t (*surface)(const Params &, const ParamsF &, const float *opsf, int mode, float dt, const StageIO &io,
-                         const float *rvol, const float *trace, cudaStream_t);
-  cudaError_t (*surfvol)(const Params &, const ParamsF &, const float *opsf, int mode, float dt, const StageIO &io,
-                         const float *rvol_in, const float *tr_in, float *rvol_out, float *tr_out, cudaStream_t);
-  int nt, epb, threads;
+  cudaError_t (*surface)(const Params &, const ParamsF &, const LineParams &, const float *opsf, int mode, float dt,
+                         const StageIO &io, const float *rvol, const float *trace, cudaStream_t);
+  cudaError_t (*surfvol)(const Params &, const ParamsF &, const LineParams &, const float *opsf, int mode, float dt,
+                         const StageIO &io, const float *rvol_in, const float *tr_in, float *rvol_out, float *tr_out,
+                         cudaStream_t);
+  int wave_tiles;  // line kernels: tiles that the GPU holds at once (stage kernel); others: 0
 };
 
 // A grid that the device holds at once is launched as a programmatic dependent
@@ -1068,7 +1076,7 @@ struct KernelSet32 {
 // balance over the SMs, so it is launched plainly (and reads with the
 // non-coherent loads, a few per cent faster on the viscous surface kernels).
 template <int P, int DIM, bool VISC, bool ST>
-cudaError_t launch_volume32(const Params &prm, const ParamsF &pf, const float *opsf, const float *w, float *rvol,
+cudaError_t launch_volume32(const Params &prm, const ParamsF &pf, const LineParams &, const float *opsf, const float *w, float *rvol,
                             float *trace, const double *w64, float *w32out, float *lo_out, double *w64copy,
                             cudaStream_t s) {
   using G = Geom<P, DIM, VISC, ST>;
@@ -1083,7 +1091,7 @@ cudaError_t launch_volume32(const Params &prm, const ParamsF &pf, const float *o
 }
 
 template <int P, int DIM, bool VISC, bool ST>
-cudaError_t launch_surface32(const Params &prm, const ParamsF &pf, const float *opsf, int mode, float dt,
+cudaError_t launch_surface32(const Params &prm, const ParamsF &pf, const LineParams &, const float *opsf, int mode, float dt,
                              const StageIO &io, const float *rvol, const float *trace, cudaStream_t s) {
   using G = Geom<P, DIM, VISC, ST>;
   const int blocks = (prm.E + G::EPB - 1) / G::EPB;
@@ -1096,7 +1104,7 @@ cudaError_t launch_surface32(const Params &prm, const ParamsF &pf, const float *
 }
 
 template <int P, int DIM, bool VISC, bool ST>
-cudaError_t launch_surfvol32(const Params &prm, const ParamsF &pf, const float *opsf, int mode, float dt,
+cudaError_t launch_surfvol32(const Params &prm, const ParamsF &pf, const LineParams &, const float *opsf, int mode, float dt,
                              const StageIO &io, const float *rvol_in, const float *tr_in, float *rvol_out,
                              float *tr_out, cudaStream_t s) {
   using G = Geom<P, DIM, VISC, ST>;
@@ -1112,10 +1120,8 @@ cudaError_t launch_surfvol32(const Params &prm, const ParamsF &pf, const float *
 
 template <int P, int DIM, bool VISC, bool ST>
 KernelSet32 make_set32() {
-  using G = Geom<P, DIM, VISC, ST>;
   return KernelSet32{&launch_volume32<P, DIM, VISC, ST>, &launch_surface32<P, DIM, VISC, ST>,
-                     &launch_surfvol32<P, DIM, VISC, ST>, VISC ? NT32_VISCOUS : NT32_INVISCID, G::EPB,
-                     G::THREADS};
+                     &launch_surfvol32<P, DIM, VISC, ST>, 0};
 }
 
 template <int P>
@@ -1133,5 +1139,7 @@ bool kernels_fp32_p(int dim, bool viscous, bool st, KernelSet32 *out) {
 }
 
 bool kernels_fp32(int p, int dim, bool viscous, bool surface_tension, KernelSet32 *out);
+// The line kernels of order p (2D, dg_lines32.cuh).
+bool lines_fp32(int p, bool viscous, bool surface_tension, KernelSet32 *out);
 
 }  // namespace dgpf
