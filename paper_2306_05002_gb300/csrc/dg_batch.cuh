@@ -25,7 +25,7 @@ namespace dgpf {
 // Everything one problem of a batch needs, read by the batched kernels from
 // device memory (one entry per problem, grouped by order).
 struct BatchProb {
-  Params prm;
+  ParamsCore prm;
   ParamsF pf;
   const float *opsf;                        // FP32 operator table (OpsLayout)
   float *ws, *d1, *d2;                      // internal FP32 state (step start) and the two inner increments

@@ -64,7 +64,7 @@ struct ParamsF {
   float rho01, rho02, drho0, mu1, mu2, sigma, gx, gy, Gamma, eps, eta_x, eta_y;
 };
 
-__host__ inline ParamsF to_float(const Params &p) {
+__host__ inline ParamsF to_float(const ParamsCore &p) {
   return ParamsF{(float)p.C2, (float)p.dC, (float)p.g1, (float)p.g2, (float)p.Bp, (float)p.rho01, (float)p.rho02,
                  (float)p.drho0, (float)p.mu1, (float)p.mu2, (float)p.sigma, (float)p.gx, (float)p.gy,
                  (float)p.Gamma, (float)p.eps, (float)p.eta_x, (float)p.eta_y};
@@ -318,7 +318,7 @@ __device__ __forceinline__ void load_line(const float *row, float *v) {
 // two derivative matrices into it unless ops_ready (the fused kernel's
 // surface part has copied the whole table and synchronised the block).
 template <int P, int DIM, bool VISC, bool ST, int EPBX = 0, bool PDL = false>
-__device__ __forceinline__ void vol32_body(const Params &prm, const ParamsF &pf, const float *__restrict__ opsf,
+__device__ __forceinline__ void vol32_body(const ParamsCore &prm, const ParamsF &pf, const float *__restrict__ opsf,
                                            float *s_op, bool ops_ready, int blk, const float *__restrict__ w,
                                            float *__restrict__ rvol, float *__restrict__ tr,
                                            const double *__restrict__ w64, float *__restrict__ w32out,
@@ -608,7 +608,7 @@ __device__ __forceinline__ void vol32_body(const Params &prm, const ParamsF &pf,
 // the kernel before (launch_dependent).
 template <int P, int DIM, bool VISC, bool ST, bool PDL>
 __global__ void __launch_bounds__(Geom<P, DIM, VISC, ST>::THREADS)
-k_volume32(const Params prm, const ParamsF pf, const float *__restrict__ opsf, const float *__restrict__ w,
+k_volume32(const ParamsCore prm, const ParamsF pf, const float *__restrict__ opsf, const float *__restrict__ w,
            float *__restrict__ rvol, float *__restrict__ tr, const double *__restrict__ w64,
            float *__restrict__ w32out, float *__restrict__ lo_out, double *__restrict__ w64copy) {
   constexpr int P11 = Geom<P, DIM, VISC, ST>::P1 * Geom<P, DIM, VISC, ST>::P1;
@@ -664,7 +664,7 @@ __device__ __forceinline__ void load_trace32(const float *__restrict__ tr, long 
 // FMAP: how face nodes are given to threads (below): 1 block-level, 0 element-level, -1 the default
 // (block-level in 2D at p = 1, 4, 5).
 template <int P, int DIM, bool VISC, bool ST, int EPBX = 0, bool PDL = false, bool FUSED = false, int FMAP = -1>
-__device__ __forceinline__ void surf32_body(const Params &prm, const ParamsF &pf, const float *__restrict__ opsf,
+__device__ __forceinline__ void surf32_body(const ParamsCore &prm, const ParamsF &pf, const float *__restrict__ opsf,
                                             float *s_op, int blk, int mode, float dt, const StageIO &io,
                                             const float *__restrict__ rvol, const float *__restrict__ tr,
                                             float *rout = nullptr) {
@@ -1010,7 +1010,7 @@ __device__ __forceinline__ void surf32_body(const Params &prm, const ParamsF &pf
 
 template <int P, int DIM, bool VISC, bool ST, bool PDL>
 __global__ void __launch_bounds__(Geom<P, DIM, VISC, ST>::THREADS)
-k_surface32(const Params prm, const ParamsF pf, const float *__restrict__ opsf, int mode, float dt, const StageIO io,
+k_surface32(const ParamsCore prm, const ParamsF pf, const float *__restrict__ opsf, int mode, float dt, const StageIO io,
             const float *__restrict__ rvol, const float *__restrict__ tr) {
   __shared__ float s_op[Geom<P, DIM, VISC, ST>::OPS];
   if (PDL) grid_dependents_launch();
@@ -1038,7 +1038,7 @@ k_surface32(const Params prm, const ParamsF pf, const float *__restrict__ opsf, 
 template <int P, int DIM, bool VISC, bool ST, bool PDL>
 __global__ void __launch_bounds__(Geom<P, DIM, VISC, ST>::THREADS,
                                   (VISC || P >= 4) ? 65536 / (Geom<P, DIM, VISC, ST>::THREADS * 72) : 1)
-k_surfvol32(const Params prm, const ParamsF pf, const float *__restrict__ opsf, int mode, float dt, const StageIO io,
+k_surfvol32(const ParamsCore prm, const ParamsF pf, const float *__restrict__ opsf, int mode, float dt, const StageIO io,
             const float *__restrict__ rvol_in, const float *__restrict__ tr_in, float *__restrict__ rvol_out,
             float *__restrict__ tr_out) {
   __shared__ float s_op[Geom<P, DIM, VISC, ST>::OPS];  // one table for both parts

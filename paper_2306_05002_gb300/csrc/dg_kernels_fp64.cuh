@@ -65,7 +65,7 @@ struct Geom {
 };
 
 // Neighbour of element e across face f (0 W, 1 E, 2 S, 3 N), or -1 at a wall.
-__device__ __forceinline__ int neighbour(const Params &p, int e, int f) {
+__device__ __forceinline__ int neighbour(const ParamsCore &p, int e, int f) {
   const int ex = e % p.nx, ey = e / p.nx;
   switch (f) {
     case 0: return ex > 0 ? e - 1 : (p.bc[0] == BC_PERIODIC ? e + p.nx - 1 : -1);
