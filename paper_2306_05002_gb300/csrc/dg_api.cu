@@ -268,7 +268,7 @@ struct dg_ctx {
   KinParams kp{};
   KinKernels kk{};
   TriKernels tk{};
-  int tri_grid = 0;
+  int tri_grid = 0, tri_epb = 1;
   double *d_kacc = nullptr, *d_kwsA = nullptr, *d_kwsB = nullptr;
   double *d_kt = nullptr, *d_kxi = nullptr, *d_ktv = nullptr;
   double *d_krvol = nullptr, *d_ktr = nullptr;  // rectangles: volume part, two buffers of face traces
@@ -1348,8 +1348,10 @@ extern "C" dg_status dg_kin_create(const dg_mesh *mesh, int p, double Gamma, dou
     int dev = 0, sms = 0, per_sm = 0;
     e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, c->tk.fn, c->tk.threads, 0);
-    const long groups = (c->E + tri_group(p) - 1) / tri_group(p);
+    c->tri_epb = c->tk.group(c->E, std::max(1, sms));
+    if (e == cudaSuccess)
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, c->tk.fn, c->tk.threads, c->tk.smem(c->tri_epb));
+    const long groups = (c->E + c->tri_epb - 1) / c->tri_epb;
     c->tri_grid = (int)std::max(1L, std::min(groups, (long)std::max(1, sms) * std::max(1, per_sm)));
   }
   if (e == cudaSuccess) e = cudaMalloc(&c->d_kt, KT_SIZE * sizeof(double));
@@ -1435,7 +1437,7 @@ extern "C" dg_status dg_kin_rhs(dg_ctx *c, const double *w, double t, double *L,
   k_kin_set_time<<<1, 4 * KIN_MAX_STEPS, 0, s>>>(c->kp, c->d_kt, t, 0.0);
   cudaError_t e = cudaGetLastError();
   if (c->tri) {
-    if (e == cudaSuccess) e = c->tk.stage(c->kp, KIN_RHS, 0, w, nullptr, nullptr, L, c->tri_grid, s);
+    if (e == cudaSuccess) e = c->tk.stage(c->kp, KIN_RHS, 0, w, nullptr, nullptr, L, c->tri_epb, c->tri_grid, s);
     return e == cudaSuccess ? DG_OK : cuda_fail(c, e, "dg_kin_rhs: launch");
   }
   if (e == cudaSuccess) e = c->kk.volume(c->kp, 0, w, c->d_krvol, c->d_ktr, s);
@@ -1458,7 +1460,7 @@ static dg_status enqueue_kin_steps(dg_ctx *c, double *w, int steps, cudaStream_t
   cudaError_t e = c->tri ? cudaSuccess : c->kk.volume(c->kp, 0, w, c->d_krvol, c->d_ktr, s);
   for (int q = 0; q < 4 * steps && e == cudaSuccess; ++q) {
     if (c->tri)
-      e = c->tk.stage(c->kp, mode[q & 3], q, in[q & 3], w, c->d_kacc, out[q & 3], c->tri_grid, s);
+      e = c->tk.stage(c->kp, mode[q & 3], q, in[q & 3], w, c->d_kacc, out[q & 3], c->tri_epb, c->tri_grid, s);
     else
       e = c->kk.stage(c->kp, mode[q & 3], q, q == 4 * steps - 1, w, c->d_kacc, c->d_krvol, c->d_ktr + (q & 1) * half,
                       c->d_ktr + (~q & 1) * half, w, s);

@@ -8,7 +8,8 @@ namespace dgpf {
 
 template <int P>
 static TriKernels tri_set() {
-  return {&launch_tri_stage<P>, &launch_tri_velocity_table<P>, (const void *)&k_tri_stage<P>, TriGeom<P>::THREADS,
+  return {&launch_tri_stage<P>, &launch_tri_velocity_table<P>, &pick_tri_epb<P>, &TriGeom<P>::smem,
+          (const void *)&k_tri_stage<P>, TriGeom<P>::THREADS,
           TriGeom<P>::NQV + TriGeom<P>::NQE};
 }
 
@@ -45,16 +46,6 @@ void tri_constants(double hx, double hy, double eta_tri, TriConst tc[2]) {
       g.gr[f] = g.rx * g.m0[f] + g.ry * g.m1[f];
       g.gs[f] = g.sx * g.m0[f] + g.sy * g.m1[f];
     }
-  }
-}
-
-int tri_group(int p) {
-  switch (p) {
-    case 1: return TriGeom<1>::EPB;
-    case 2: return TriGeom<2>::EPB;
-    case 3: return TriGeom<3>::EPB;
-    case 4: return TriGeom<4>::EPB;
-    default: return 0;
   }
 }
 

@@ -17,8 +17,8 @@
 // a_1 with its symmetric term, penalty eta = c_ip (p+1)(p+2) / h_e with
 // h_e = 2 |T| / |e|.
 //
-// One kernel per Runge-Kutta stage.  A persistent grid walks groups of EPB
-// triangles; each CTA stages the reference tables (basis values and
+// One kernel per Runge-Kutta stage.  A persistent grid walks groups of epb
+// triangles (pick_tri_epb); each CTA stages the reference tables (basis values and
 // derivatives at the volume and edge points, the inverse reference mass matrix)
 // in shared memory once, then per group: the own and neighbour nodal values,
 // the integrand coefficients at every volume and edge point (one thread per
@@ -81,8 +81,12 @@ template <int P>
 struct TriGeom {
   static constexpr TriLayout L{P};
   static constexpr int NP = L.NP, NQ1 = L.NQ1, NQV = L.NQV, NQE = L.NQE;
-  static constexpr int EPB = P >= 4 ? 6 : 8;
-  static constexpr int THREADS = 128;
+  static constexpr int THREADS = 256;
+  // shared memory in doubles: the tables; per triangle its own and its neighbours' values, the
+  // coefficients at its volume and edge points, its weak-form sums
+  static constexpr int PER = 10 * NP + 4 * (NQV + NQE);
+  static constexpr size_t smem(int epb) { return sizeof(double) * (L.size() + (size_t)epb * PER); }
+  static constexpr int MAX_EPB = (int)((48 * 1024 / sizeof(double) - L.size()) / PER);
 };
 
 
@@ -214,35 +218,59 @@ __device__ __forceinline__ void tri_edge_trace(const double *s_t, const TriLayou
   o->n_m = has_gradient(g2) ? sgn * gs * rsqrt64(g2) : 0.0;  // n = 0 where |grad psi| < 1e-12
 }
 
+// Triangles per group: the count with the least FP64 work on the SM that has the most, where a phase costs
+// the warps that its items fill (volume points, edge points, nodes) times the operations of one; ties go
+// to the larger group (fewer copies of the tables).  2,048 triangles at p = 3: 14, one group on each of 147
+// SMs and nearly full warps, 28.0 us a stage against 31.8 in groups of 8, two on most SMs and
+// one on the others.
+template <int P>
+int pick_tri_epb(int E, int sms) {
+  using G = TriGeom<P>;
+  constexpr int NP = G::NP, NQ1 = G::NQ1, NQV = G::NQV, NQE = G::NQE;
+  constexpr long CV = 10 * NP + 45, CE = 6 * (P + 1) + 4 * NP + 25, CN = 8 * NQV + 2 * NQE + 4 * NQ1 + 4 * NP;
+  int best = 1;
+  long best_cost = 0;
+  for (int epb = 1; epb <= G::MAX_EPB && epb <= 32; ++epb) {
+    const auto warps = [epb](int items) { return (long)(epb * items + 31) / 32; };
+    const long groups = ((long)E + epb - 1) / epb;
+    const long cost = (groups + sms - 1) / sms * (CV * warps(NQV) + CE * warps(NQE) + CN * warps(NP));
+    if (epb == 1 || cost <= best_cost) {
+      best = epb;
+      best_cost = cost;
+    }
+  }
+  return best;
+}
+
 // One stage: the right-hand side L = M^-1 R(win) at the time of stage ic of the
 // captured sequence (KinTime), written as L (KIN_RHS) or as one classical RK4 stage (KIN_K1..K4, the same
 // updates as k_kin_stage; out may be w0, each node being read, then written,
 // by the same thread).
 template <int P>
 __global__ void __launch_bounds__(TriGeom<P>::THREADS)
-k_tri_stage(const KinParams kp, int mode, int ic, const double *__restrict__ win, const double *w0,
+k_tri_stage(const KinParams kp, int epb, int mode, int ic, const double *__restrict__ win, const double *w0,
             double *__restrict__ acc, double *out) {
   using G = TriGeom<P>;
   constexpr TriLayout L = G::L;
-  constexpr int NP = G::NP, NQ1 = G::NQ1, NQV = G::NQV, NQE = G::NQE, EPB = G::EPB;
+  constexpr int NP = G::NP, NQ1 = G::NQ1, NQV = G::NQV, NQE = G::NQE;
   constexpr int NPT = NQV + NQE;
-  __shared__ double s_t[L.size()];
-  __shared__ double s_w[EPB][2][NP];
-  __shared__ double s_nb[EPB][3][2][NP];
-  __shared__ double s_cv[EPB][NQV][4];
-  __shared__ double s_ce[EPB][NQE][4];
-  __shared__ double s_R[EPB][2][NP];
+  extern __shared__ double s_tri[];
+  double *const s_t = s_tri;
+  double(*const s_w)[4][2][NP] = reinterpret_cast<double(*)[4][2][NP]>(s_t + L.size());  // own, neighbours
+  double(*const s_cv)[NQV][4] = reinterpret_cast<double(*)[NQV][4]>(s_w + epb);
+  double(*const s_ce)[NQE][4] = reinterpret_cast<double(*)[NQE][4]>(s_cv + epb);
+  double(*const s_R)[2][NP] = reinterpret_cast<double(*)[2][NP]>(s_ce + epb);
   for (int i = threadIdx.x; i < L.size(); i += blockDim.x) s_t[i] = kp.ops[i];
   const double c = kp.kt[KT_C + ic];
   const double hstep = kp.kt[mode == KIN_K4 ? KT_SIXTH : (mode == KIN_K3 ? KT_DT : KT_HALF)];
-  const int N = kp.N, ngroups = (kp.E + EPB - 1) / EPB;
+  const int N = kp.N, ngroups = (kp.E + epb - 1) / epb;
   bool bad = false;
 
   for (int grp = blockIdx.x; grp < ngroups; grp += gridDim.x) {
-    const int e0 = grp * EPB;
+    const int e0 = grp * epb;
     __syncthreads();  // tables staged; the previous group's shared data consumed
     // 1. Own (slot 0) and neighbour (slots 1..3) nodal values.
-    for (int it = threadIdx.x; it < EPB * 4 * NP; it += blockDim.x) {
+    for (int it = threadIdx.x; it < epb * 4 * NP; it += blockDim.x) {
       const int n = it % NP, slot = (it / NP) % 4, le = it / (4 * NP), e = e0 + le;
       double a = 0.0, b = 0.0;
       if (e < kp.E) {
@@ -253,19 +281,19 @@ k_tri_stage(const KinParams kp, int mode, int ic, const double *__restrict__ win
           b = win[N + (long)src * NP + n];
         }
       }
-      double *dst = slot == 0 ? s_w[le][0] : s_nb[le][slot - 1][0];
+      double *dst = s_w[le][slot][0];
       dst[n] = a;
       dst[NP + n] = b;
     }
     __syncthreads();
     // 2. Volume points: coefficients of l_n, dl_n/dr, dl_n/ds (phi) and l_n (psi).
-    for (int it = threadIdx.x; it < EPB * NQV; it += blockDim.x) {
+    for (int it = threadIdx.x; it < epb * NQV; it += blockDim.x) {
       const int le = it / NQV, q = it % NQV, e = e0 + le;
       double cv[4] = {0.0, 0.0, 0.0, 0.0};
       if (e < kp.E) {
         const TriConst &g = kp.tc[e & 1];
         TriPoint o;
-        tri_eval_point<NP, false>(kp, g, s_w[le][0], s_w[le][1], s_t + L.bv() + q * NP, s_t + L.brv() + q * NP,
+        tri_eval_point<NP, false>(kp, g, s_w[le][0][0], s_w[le][0][1], s_t + L.bv() + q * NP, s_t + L.brv() + q * NP,
                            s_t + L.bsv() + q * NP, &o);
         const long ov = (long)e * NPT + q;
         const double2 U = in_bounds(kp.status, ov, (long long)kp.E * NPT)
@@ -284,7 +312,7 @@ k_tri_stage(const KinParams kp, int mode, int ic, const double *__restrict__ win
     // 3. Edge points: transport and SIP fluxes, the symmetric term.  On each side: phi and psi
     //    from the p+1 edge nodes, the normal derivatives of phi and psi from all nodes (bn), the
     //    tangential derivative of psi from the edge nodes -- n . m = (d psi/dm) / |grad psi|.
-    for (int it = threadIdx.x; it < EPB * NQE; it += blockDim.x) {
+    for (int it = threadIdx.x; it < epb * NQE; it += blockDim.x) {
       const int le = it / NQE, fk = it % NQE, f = fk / NQ1, k = fk % NQ1, e = e0 + le;
       double ce[4] = {0.0, 0.0, 0.0, 0.0};
       if (e < kp.E) {
@@ -293,8 +321,8 @@ k_tri_stage(const KinParams kp, int mode, int ic, const double *__restrict__ win
         const int fk2 = f2 * NQ1 + (NQ1 - 1 - k);  // the same physical point, seen from the neighbour
         const TriConst &g = kp.tc[e & 1], &g2 = kp.tc[e2 & 1];
         TriEdgeTrace om, op;
-        tri_edge_trace<P>(s_t, L, e & 1, f, fk, s_w[le][0], s_w[le][1], g.ihl[f], 1.0, &om);
-        tri_edge_trace<P>(s_t, L, e2 & 1, f2, fk2, s_nb[le][f][0], s_nb[le][f][1], g2.ihl[f2], -1.0, &op);
+        tri_edge_trace<P>(s_t, L, e & 1, f, fk, s_w[le][0][0], s_w[le][0][1], g.ihl[f], 1.0, &om);
+        tri_edge_trace<P>(s_t, L, e2 & 1, f2, fk2, s_w[le][1 + f][0], s_w[le][1 + f][1], g2.ihl[f2], -1.0, &op);
         const double2 *vt = reinterpret_cast<const double2 *>(kp.vel_tab);
         const long vm = (long)e * NPT + NQV + fk, vp = (long)e2 * NPT + NQV + fk2;
         const long long nt = (long long)kp.E * NPT;
@@ -319,7 +347,7 @@ k_tri_stage(const KinParams kp, int mode, int ic, const double *__restrict__ win
     __syncthreads();
     // 4. Weak-form sums R_n: volume points, the lifted symmetric term at every edge point, and
     //    the edge fluxes at the edges the node lies on.
-    for (int it = threadIdx.x; it < EPB * NP; it += blockDim.x) {
+    for (int it = threadIdx.x; it < epb * NP; it += blockDim.x) {
       const int le = it / NP, n = it % NP;
       double rp = 0.0, rs = 0.0;
 #pragma unroll 4
@@ -356,7 +384,7 @@ k_tri_stage(const KinParams kp, int mode, int ic, const double *__restrict__ win
     }
     __syncthreads();
     // 5. L = M^-1 R / det and the stage update.
-    for (int it = threadIdx.x; it < EPB * NP; it += blockDim.x) {
+    for (int it = threadIdx.x; it < epb * NP; it += blockDim.x) {
       const int le = it / NP, n = it % NP, e = e0 + le;
       if (e >= kp.E || !in_bounds(kp.status, (long)e * NP + n, N)) continue;
       const double idet = kp.tc[e & 1].idet;
@@ -392,8 +420,10 @@ k_tri_stage(const KinParams kp, int mode, int ic, const double *__restrict__ win
 
 struct TriKernels {
   cudaError_t (*stage)(const KinParams &, int mode, int ic, const double *win, const double *w0, double *acc,
-                       double *out, int grid, cudaStream_t);
+                       double *out, int epb, int grid, cudaStream_t);
   cudaError_t (*velocity_table)(const KinParams &, double *tab, cudaStream_t);
+  int (*group)(int E, int sms);  // triangles per group (pick_tri_epb)
+  size_t (*smem)(int epb);       // dynamic shared memory of the stage kernel
   const void *fn;  // the stage kernel, for the occupancy query
   int threads;
   int points;      // volume + edge points per triangle (rows of the velocity table)
@@ -401,15 +431,13 @@ struct TriKernels {
 
 template <int P>
 cudaError_t launch_tri_stage(const KinParams &kp, int mode, int ic, const double *win, const double *w0, double *acc,
-                             double *out, int grid, cudaStream_t s) {
-  k_tri_stage<P><<<grid, TriGeom<P>::THREADS, 0, s>>>(kp, mode, ic, win, w0, acc, out);
+                             double *out, int epb, int grid, cudaStream_t s) {
+  k_tri_stage<P><<<grid, TriGeom<P>::THREADS, TriGeom<P>::smem(epb), s>>>(kp, epb, mode, ic, win, w0, acc, out);
   return cudaGetLastError();
 }
 
 // Kernels of order p (1..4); false for other orders.
 bool tri_kernels(int p, TriKernels *out);
-// Triangles one CTA processes per pass (EPB of order p).
-int tri_group(int p);
 // Tables of order p in the TriLayout order, the normal derivatives for the two triangle types
 // of constants tc; empty on failure.
 std::vector<double> tri_tables(int p, const TriConst tc[2]);
