@@ -16,10 +16,19 @@
 //     their own.
 //   * the face records and the volume part are all requested before the first flux is formed.
 // It executes less than half of the instructions per node of the one-node-per-thread kernels (p = 4,
-// viscous, surface tension: 700 instead of 1,560; no index arithmetic or divisions per face node, no
+// viscous, surface tension: 780 instead of 1,560; no index arithmetic or divisions per face node, no
 // shared load per term), which is what bounds those on grids of many waves, but a thread's chain is
 // P + 1 times as long and a warp holds four to six times the nodes, so a mesh that does not fill the
 // GPU is left to the one-node-per-thread kernels (use_lines32).
+// Measured, 10 steps of a viscous Rayleigh-Taylor problem with surface tension, 256 x 256, p = 4: 3082 us one
+// node per thread, 2795 here.  What bounds them is instruction issue with exposed load latency, at 12 warps
+// an SM.
+//
+// Every operation is rounded as in the one-node-per-thread kernels (see face_flux32), so that the same
+// problem does not change its result with its size class.  Grouping the momentum and energy terms saves
+// another 2%, but turns last bits of the FP32-rounded phase field, 9e-8 at single nodes after four steps.
+// Batches keep one node per thread: on these kernels the mixed ensembles measured 7 to 15% slower, and
+// small ones up to twice as slow.
 #pragma once
 
 #include "dg_kernels_fp32.cuh"
@@ -51,7 +60,7 @@ struct LineParams {
   float p_bc[4];
   float eta_x, eta_y;
   float C2, dC, g2, dg, Bp;
-  float rho01, rho02, drho0, hdr, mu2, dmu, sigma, gx, gy, Gamma, eps;
+  float rho01, rho02, drho0, mu2, dmu, sigma, gx, gy, Gamma, eps;
   int gravity, check_finite;
   double C2d, dCd;
   unsigned *status;
@@ -81,7 +90,6 @@ __host__ inline LineParams line_params(const Params &p, int P1, const float *ops
   f.rho01 = (float)p.rho01;
   f.rho02 = (float)p.rho02;
   f.drho0 = (float)p.drho0;
-  f.hdr = 0.5f * (float)p.drho0;
   f.mu2 = (float)p.mu2;
   f.dmu = (float)p.mu1 - (float)p.mu2;
   f.sigma = (float)p.sigma;
@@ -284,7 +292,6 @@ __device__ __forceinline__ void ld_trace(const float4 *__restrict__ tr, int E, u
   }
 }
 
-#define FACE_LF(dF, lam, dw) fmaf((lam) * 0.5f, dw, 0.5f * (dF))
 // ---------------------------------------------------------------------------
 // Face flux
 // ---------------------------------------------------------------------------
@@ -355,7 +362,7 @@ __device__ __forceinline__ void face_flux32(const LineParams &pf, const float *t
       const float dF = (XF ? c == 2 : c == 3) ? Fm[c] - Fp[c]
                        : c == 4               ? fmaf(tm[RE] + m.P, unm, -Fp[4])
                                               : fmaf(tm[v], unm, -Fp[c]);
-      S[v] = wf * FACE_LF(dF, lam, tp[v] - tm[v]);
+      S[v] = wf * fmaf(lam * 0.5f, tp[v] - tm[v], 0.5f * dF);
     }
   }
   // compression term on the face: -1/2 Cmix(phi+) (u+ - u-) . m
