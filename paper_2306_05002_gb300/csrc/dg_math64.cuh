@@ -87,8 +87,8 @@ __device__ __forceinline__ double sqrt64(double x) {
 
 // The correctly rounded forms: a residual step on the third-order result (Markstein: with y within
 // a unit of 1 / b, fma(y, fma(-b, y, 1), y) is the rounded reciprocal, and fma(r, y, q), q = a y and
-// r = a - b q, the rounded quotient; likewise for the square root with y / 2 = 1 / (2 sqrt(x))).
-// A quotient then costs three operations after its denominator's five.
+// r = a - b q, the rounded quotient).  A quotient then costs three operations after its denominator's
+// five.
 // The theorem's one exception is a denominator whose significand is all ones, e.g. 1 - 2^-53 (which a
 // sum of partial densities can be): CUDA's division takes it.
 __device__ __forceinline__ double rcp64_rn(double x) {
@@ -109,14 +109,23 @@ __device__ __forceinline__ double div64_rn(double a, double b, double y) {
   return fma(fma(-b, q, a), y, q);
 }
 
+// sqrt(x), correctly rounded: s = t (1 + d), t = x y and d = e / 2 + 3 e^2 / 8 (sqrt64), then the
+// residual step s + (x - s^2) / (2 sqrt(x)).  Its multiplier has to be good to about a unit in the last
+// place, so it is y (1 + d) / 2, not y / 2.  With u = 2^-53: the rounding of t moves s and y (1 + d) by
+// u / 2, so s is within a unit of the root, x - s^2 is exact, and the multiplier is off by at most 3 u / 2
+// (its own rounding included), the correction, half a unit near a boundary S + 1/2, by less than 3 u / 4 of a
+// unit.  The root nearest to a boundary has x = S^2 + S + j with a small j, and j is even: for |j| >= 2 the
+// distance is at least 7 / (8 S), of which the step's second order takes 1 / (8 S), which leaves more than
+// 3 u / 4.  j = 0 only for 1 - 2^-53 and 1 + 2^-52 times powers of four, both rounded right.
 __device__ __forceinline__ double sqrt64_rn(double x) {
   if (!mid_range64(x)) return sqrt64_slow(x);
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
   const double t = x * y;
   const double e = fma(-t, y, 1.0);
-  const double s = fma(t * e, fma(e, 0.375, 0.5), t);
-  const double h = __hiloint2double(__double2hiint(y) - 0x100000, __double2loint(y));  // y / 2
+  const double d = e * fma(e, 0.375, 0.5);
+  const double s = fma(t, d, t), r = fma(y, d, y);
+  const double h = __hiloint2double(__double2hiint(r) - 0x100000, __double2loint(r));  // r / 2
   return fma(fma(-s, s, x), h, s);
 }
 
