@@ -43,6 +43,12 @@ __device__ __forceinline__ bool has_gradient(double g2) {
   return b >= __double_as_longlong(1e-24) && b <= 0x7ff0000000000000ll;
 }
 
+// x < 1e-24 for x >= 0 or NaN (false for a NaN), without an FP64 comparison: the same cut-off where a NaN
+// has to stay one.
+__device__ __forceinline__ bool no_gradient(double g2) {
+  return (unsigned long long)__double_as_longlong(g2) < (unsigned long long)__double_as_longlong(1e-24);
+}
+
 // Exponents for which the iterations below neither overflow nor lose bits to gradual underflow:
 // 2^-500 .. 2^500.  Zeros, infinities, NaNs, subnormals and everything outside go to CUDA's own
 // functions (never in a physical state; the branch is not taken).

@@ -173,7 +173,7 @@ __device__ __forceinline__ void tri_eval_point(const KinParams &kp, const TriCon
   o->gs[0] = sr * g.rx + sq * g.sx;
   o->gs[1] = sr * g.ry + sq * g.sy;
   const double g2 = o->gs[0] * o->gs[0] + o->gs[1] * o->gs[1];
-  const double rn = has_gradient(g2) ? rsqrt64(g2) : 0.0;  // n = 0 where |grad psi| < 1e-12
+  const double rn = no_gradient(g2) ? 0.0 : rsqrt64(g2);  // n = 0 where |grad psi| < 1e-12
   const double sp = ph * (1.0 - ph);
 #pragma unroll
   for (int d = 0; d < 2; ++d) {
@@ -215,7 +215,7 @@ __device__ __forceinline__ void tri_edge_trace(const double *s_t, const TriLayou
   o->phi = ph;
   o->psi = ps;
   o->dphi_m = sgn * gp;
-  o->n_m = has_gradient(g2) ? sgn * gs * rsqrt64(g2) : 0.0;  // n = 0 where |grad psi| < 1e-12
+  o->n_m = no_gradient(g2) ? 0.0 : sgn * gs * rsqrt64(g2);  // n = 0 where |grad psi| < 1e-12
 }
 
 // Triangles per group: the count with the least FP64 work on the SM that has the most, where a phase costs
