@@ -179,10 +179,18 @@ __device__ __forceinline__ void kin_volume_part(const KinParams &kp, const doubl
     gpy = k ? fma(dy, s_f[sy + P1 * k], gpy) : dy * s_f[sy];
     gsy = k ? fma(dy, s_f[fs + sy + P1 * k], gsy) : dy * s_f[fs + sy];
   }
-  // a_1 = Gamma (eps grad phi - phi (1 - phi) grad psi / |grad psi|), n = 0 where |grad psi| < 1e-12
+  // a_1 = Gamma (eps grad phi - phi (1 - phi) grad psi / |grad psi|), n = 0 unless |grad psi| >= 1e-12 (so a
+  // NaN there does not reach phi)
   const double g2 = fma(gsy, gsy, gsx * gsx);
-  const double Gn = has_gradient(g2) ? kp.Gamma * fma(-phi, phi, phi) * rsqrt64(g2) : 0.0;
-  const double a1x = fma(kp.Ge, gpx, -(Gn * gsx)), a1y = fma(kp.Ge, gpy, -(Gn * gsy));
+  double a1x, a1y;
+  if (has_gradient(g2)) {
+    const double Gn = kp.Gamma * fma(-phi, phi, phi) * rsqrt64(g2);
+    a1x = fma(kp.Ge, gpx, -(Gn * gsx));
+    a1y = fma(kp.Ge, gpy, -(Gn * gsy));
+  } else {
+    a1x = kp.Ge * gpx;
+    a1y = kp.Ge * gpy;
+  }
   __syncthreads();
   if (lane) {
     s_f[sn] = a1x;

@@ -3,7 +3,8 @@ is not.
 
 On triangles n = grad psi / |grad psi| is taken as zero where |grad psi| < 1e-12, which a NaN is not, so
 the NaN reaches the phase field through the normals of the triangle and of its neighbours' edges, as in
-the oracle.  psi itself is NaN and the status word says so."""
+the oracle.  On rectangles n is zero unless |grad psi| >= 1e-12: the phase field's right-hand side stays
+what the finite part of the state gives.  Either way psi itself is NaN and the status word says so."""
 import numpy as np
 import pytest
 
@@ -39,3 +40,19 @@ def test_nan_level_set_on_triangles(orc, dg, p):
     # (the edges read psi at their own nodes alone, the oracle at all of the element's)
     assert nan[1].any() and not (nan[1] & ~ref[1]).any()
     assert status == -5  # DG_ERR_NONFINITE
+
+
+@pytest.mark.parametrize("p", [1, 2, 3, 4, 5])
+def test_nan_level_set_on_rectangles(dg, p):
+    wl = W.rider_kothe(n=6, p=p)
+    Np = (p + 1) ** 2
+    w = wl.w.copy()
+    w[1, 14 * Np + Np // 2] = np.nan
+    L, status = _rhs(dg, wl, w)
+    L0, _ = _rhs(dg, wl, wl.w.copy())
+    assert np.isfinite(L[0]).all() and np.isnan(L[1]).any()
+    far = np.ones(wl.N, bool)  # elements that neither hold nor touch the node
+    for e in (14, 13, 15, 8, 20):
+        far[e * Np:(e + 1) * Np] = False
+    assert np.array_equal(L[:, far], L0[:, far])
+    assert status == -5
