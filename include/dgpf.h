@@ -226,10 +226,11 @@ const char *dg_last_error(const dg_ctx *ctx);
    the mean duration per launch in milliseconds to ms_out
    (index 0 volume kernel, 1 surface kernel, and for FP32-bulk contexts 2 the
    fused kernel that dg_step runs: the surface part of one stage followed by
-   the volume part of the next, 3 the volume kernel of a call's first stage,
-   which reads the FP64 state, and 4 the surface kernel of a call's last
-   stage, which writes it -- into a temporary FP64 array that this call
-   allocates and frees); returns the number of kinds written (<= nmax), or
+   the volume part of the next, all three as in a sequence of eight steps, and
+   of a call of one step 3 the volume kernel of its first stage, which reads
+   the FP64 state, and 4 the surface kernel of its last stage, which writes it
+   -- into a temporary FP64 array that this call allocates and frees); returns
+   the number of kinds written (<= nmax), or
    -1.  w is not modified.  Synchronises the stream. */
 int dg_time_kernels(dg_ctx *ctx, const double *w, int nrep, double *ms_out, int nmax, void *stream);
 
@@ -240,6 +241,12 @@ int dg_time_kernels(dg_ctx *ctx, const double *w, int nrep, double *ms_out, int 
    stage one fused surface + next-volume kernel, the last stage's surface
    kernel alone).  -1 for a NULL, batch or kinematic context or nsteps < 0. */
 int dg_step_launches(const dg_ctx *ctx, int nsteps);
+
+/* Which FP32-bulk kernels a call runs on this context: 1 when a dg_step call
+   of nsteps steps (0: a dg_rhs call; more than 8: its sequences of eight) runs
+   those with one element line per thread, 0 when those with one node per
+   thread (or FP64).  -1 for a NULL, batch or kinematic context or nsteps < 0. */
+int dg_line_kernels(const dg_ctx *ctx, int nsteps);
 
 /* Algorithmic FP64-equivalent flop and DRAM byte counts per launch of each
    kernel kind (same indexing as dg_time_kernels), from the formulas of the

@@ -249,8 +249,10 @@ struct dg_ctx {
   KernelSet ks;
   KernelSet32 ks32;
   ParamsF pf;
-  LineParams lp{};      // FP32-bulk, 2D: the line kernels' parameters
-  bool lines = false;   // FP32-bulk: this context runs the line kernels (use_lines32)
+  // FP32-bulk, 2D: the line kernels, their parameters and the calls that run them (use_lines32)
+  KernelSet32 ksl{};
+  LineParams lp{};
+  LineUse lu{false, 0};
   int prec = DG_FP64;
   AdjKernels adj{};
   bool has_adj = false;
@@ -457,13 +459,15 @@ extern "C" dg_status dg_create(const dg_mesh *mesh, int p, const dg_eos *eos, do
     return e == cudaSuccess;
   };
   if (!f64) {
-    KernelSet32 kl;
-    c->lines = c->dim == 2 && lines_fp32(p, o.viscous != 0, o.surface_tension != 0, &kl) &&
-               use_lines32(P1, o.viscous || o.surface_tension, c->E, kl.wave_tiles);
-    if (c->lines) c->ks32 = kl;
-    // one padded record per node (inviscid kernels) and per face node, or the line kernels' tiles
-    const size_t n32 = c->lines ? line_node_floats(P1, c->E) : (size_t)SW32 * c->N;
-    const size_t t32 = c->lines ? line_trace_floats(P1, c->E) : (size_t)TRW32 * c->E * c->NFK;
+    if (c->dim == 2 && lines_fp32(p, o.viscous != 0, o.surface_tension != 0, &c->ksl))
+      c->lu = use_lines32(P1, o.viscous != 0, o.surface_tension != 0, c->E, c->ks32, c->ksl);
+    // one padded record per node (inviscid kernels) and per face node, and room for the line kernels' tiles:
+    // every call writes what it reads, so calls on either layout share the arrays
+    size_t n32 = (size_t)SW32 * c->N, t32 = (size_t)TRW32 * c->E * c->NFK;
+    if (c->lu.rhs || c->lu.steps) {
+      n32 = std::max(n32, line_node_floats(P1, c->E));
+      t32 = std::max(t32, line_trace_floats(P1, c->E));
+    }
     c->n32 = n32;
     alloc32(&c->d_opsf, opsf.size()) && alloc32(&c->d_hi32[0], n32) && alloc32(&c->d_hi32[1], n32) &&
         alloc32(&c->d_lo32[0], n32) && alloc32(&c->d_lo32[1], n32) && alloc32(&c->d_dd32[0], n32) &&
@@ -497,7 +501,7 @@ extern "C" dg_status dg_create(const dg_mesh *mesh, int p, const dg_eos *eos, do
   }
   q.ops = c->d_ops;
   q.status = c->d_status;
-  if (c->lines) c->lp = line_params(c->prm, P1, opsf.data(), c->d_opsf);
+  if (c->lu.rhs || c->lu.steps) c->lp = line_params(c->prm, P1, opsf.data(), c->d_opsf);
   *out = c;
   return DG_OK;
 }
@@ -585,15 +589,27 @@ static dg_status run_stage(dg_ctx *c, int mode, double dt, const double *w0, con
   return DG_OK;
 }
 
+// The FP32-bulk kernels of a captured sequence of `steps` steps (0: of a right-hand side).
+static bool runs_lines(const dg_ctx *c, int steps) {
+  return steps == 0 ? c->lu.rhs : c->lu.steps > 0 && steps >= c->lu.steps;
+}
+static const KernelSet32 &set32(const dg_ctx *c, int steps) { return runs_lines(c, steps) ? c->ksl : c->ks32; }
+
+extern "C" int dg_line_kernels(const dg_ctx *c, int nsteps) {
+  if (!c || c->batch || c->kin || nsteps < 0) return -1;
+  return c->prec != DG_FP64 && runs_lines(c, std::min(nsteps, GRAPH_UNROLL));
+}
+
 // The FP32-bulk right-hand side of the FP64 state w64: the volume kernel splits
 // the state into the internal hi part (the lo part is not needed) and the
 // surface kernel writes L in FP64.
 static dg_status rhs32(dg_ctx *c, const double *w64, double *L, cudaStream_t s) {
-  cudaError_t e = c->ks32.volume(c->prm, c->pf, c->lp, c->d_opsf, nullptr, c->d_rvol32, c->d_trace32, w64, c->d_hi32[0],
+  const KernelSet32 &ks = set32(c, 0);
+  cudaError_t e = ks.volume(c->prm, c->pf, c->lp, c->d_opsf, nullptr, c->d_rvol32, c->d_trace32, w64, c->d_hi32[0],
                                  nullptr, nullptr, s);
   if (e != cudaSuccess) return cuda_fail(c, e, "volume kernel launch");
   const StageIO io{nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, L, nullptr};
-  e = c->ks32.surface(c->prm, c->pf, c->lp, c->d_opsf, MODE_RHS, 0.f, io, c->d_rvol32, c->d_trace32, s);
+  e = ks.surface(c->prm, c->pf, c->lp, c->d_opsf, MODE_RHS, 0.f, io, c->d_rvol32, c->d_trace32, s);
   if (e != cudaSuccess) return cuda_fail(c, e, "surface kernel launch");
   return DG_OK;
 }
@@ -640,10 +656,11 @@ static dg_status enqueue_steps32(dg_ctx *c, double *w, float dt, int steps, cuda
                                  double *copy64 = nullptr) {
   float *const *H = c->d_hi32, *const *Lo = c->d_lo32, *const *D = c->d_dd32;
   float *rv[2] = {c->d_rvol32, c->d_rvol32b}, *tr[2] = {c->d_trace32, c->d_trace32b};
+  const KernelSet32 &ks = set32(c, steps);
   int t = 0, a = 0;
   if (steps != 1) copy64 = nullptr;
   // a single step adds its last increment to the FP64 state itself: no lo part is needed
-  cudaError_t e = c->ks32.volume(c->prm, c->pf, c->lp, c->d_opsf, nullptr, rv[t], tr[t], w, H[a], steps > 1 ? Lo[a] : nullptr,
+  cudaError_t e = ks.volume(c->prm, c->pf, c->lp, c->d_opsf, nullptr, rv[t], tr[t], w, H[a], steps > 1 ? Lo[a] : nullptr,
                                  copy64, s);
   if (e != cudaSuccess) return cuda_fail(c, e, "volume kernel launch");
   for (int k = 0; k < steps; ++k) {
@@ -656,11 +673,11 @@ static dg_status enqueue_steps32(dg_ctx *c, double *w, float dt, int steps, cuda
     const int mode[3] = {MODE_S1, MODE_S2, MODE_S3};
     for (int st = 0; st < 3; ++st) {
       if (st == 2 && last) {
-        e = c->ks32.surface(c->prm, c->pf, c->lp, c->d_opsf, MODE_S3, dt, io[2], rv[t], tr[t], s);
+        e = ks.surface(c->prm, c->pf, c->lp, c->d_opsf, MODE_S3, dt, io[2], rv[t], tr[t], s);
         if (e != cudaSuccess) return cuda_fail(c, e, "surface kernel launch");
         break;
       }
-      e = c->ks32.surfvol(c->prm, c->pf, c->lp, c->d_opsf, mode[st], dt, io[st], rv[t], tr[t], rv[t ^ 1], tr[t ^ 1], s);
+      e = ks.surfvol(c->prm, c->pf, c->lp, c->d_opsf, mode[st], dt, io[st], rv[t], tr[t], rv[t ^ 1], tr[t ^ 1], s);
       if (e != cudaSuccess) return cuda_fail(c, e, "fused stage kernel launch");
       t ^= 1;
     }
@@ -835,6 +852,7 @@ extern "C" int dg_time_kernels(dg_ctx *c, const double *w, int nrep, double *ms_
   cudaStream_t s = (cudaStream_t)stream;
   const bool f64 = c->prec == DG_FP64;
   const int nk = f64 ? 2 : 5;
+  const KernelSet32 &kq = set32(c, GRAPH_UNROLL), &k1 = set32(c, 1);  // of long sequences, of a single step
   // FP32-bulk kind 4 writes an FP64 state: into a temporary, not the caller's w
   double *tmp64 = nullptr;
   if (!f64 && nmax > 4 && cudaMalloc(&tmp64, c->len * sizeof(double)) != cudaSuccess) {
@@ -849,25 +867,25 @@ extern "C" int dg_time_kernels(dg_ctx *c, const double *w, int nrep, double *ms_
       if (k == 0) c->ks.volume(c->prm, w, c->d_rvol, c->d_trace, s);
       else c->ks.surface(c->prm, MODE_RHS, 0.0, w, w, c->d_rvol, c->d_trace, c->d_w1, s);
     } else if (k == 0) {  // the kernels of a step as dg_step launches them (FP32 state in, FP32 stage out)
-      c->ks32.volume(c->prm, c->pf, c->lp, c->d_opsf, c->d_hi32[0], c->d_rvol32, c->d_trace32, nullptr, nullptr, nullptr,
+      kq.volume(c->prm, c->pf, c->lp, c->d_opsf, c->d_hi32[0], c->d_rvol32, c->d_trace32, nullptr, nullptr, nullptr,
                      nullptr, s);
     } else if (k == 1) {
       const StageIO io{c->d_hi32[0], nullptr, c->d_dd32[0], c->d_dd32[1], nullptr, nullptr, nullptr, nullptr};
-      c->ks32.surface(c->prm, c->pf, c->lp, c->d_opsf, MODE_S2, 1e-9f, io, c->d_rvol32, c->d_trace32, s);
+      kq.surface(c->prm, c->pf, c->lp, c->d_opsf, MODE_S2, 1e-9f, io, c->d_rvol32, c->d_trace32, s);
     } else if (k == 2) {
       const StageIO io{c->d_hi32[0], nullptr, c->d_dd32[0], c->d_dd32[1], nullptr, nullptr, nullptr, nullptr};
-      c->ks32.surfvol(c->prm, c->pf, c->lp, c->d_opsf, MODE_S2, 1e-9f, io, c->d_rvol32, c->d_trace32, c->d_rvol32b,
+      kq.surfvol(c->prm, c->pf, c->lp, c->d_opsf, MODE_S2, 1e-9f, io, c->d_rvol32, c->d_trace32, c->d_rvol32b,
                       c->d_trace32b, s);
     } else if (k == 3) {  // the first stage of a single-step call: reads the FP64 state (hi part only)
-      c->ks32.volume(c->prm, c->pf, c->lp, c->d_opsf, nullptr, c->d_rvol32b, c->d_trace32b, w, c->d_hi32[1], nullptr,
+      k1.volume(c->prm, c->pf, c->lp, c->d_opsf, nullptr, c->d_rvol32b, c->d_trace32b, w, c->d_hi32[1], nullptr,
                      nullptr, s);
-    } else {  // the last stage of a single-step call: adds the last increment to the FP64 state
+    } else {  // the last stage of a single-step call, after kind 3: adds the last increment to the FP64 state
       const StageIO io{nullptr, nullptr, c->d_dd32[0], nullptr, nullptr, nullptr, tmp64, w};
-      c->ks32.surface(c->prm, c->pf, c->lp, c->d_opsf, MODE_S3, 1e-9f, io, c->d_rvol32, c->d_trace32, s);
+      k1.surface(c->prm, c->pf, c->lp, c->d_opsf, MODE_S3, 1e-9f, io, c->d_rvol32b, c->d_trace32b, s);
     }
   };
   if (!f64) {  // the internal state of w (hi, lo) and a zero increment to time the stage kernels on
-    c->ks32.volume(c->prm, c->pf, c->lp, c->d_opsf, nullptr, c->d_rvol32, c->d_trace32, w, c->d_hi32[0], c->d_lo32[0],
+    kq.volume(c->prm, c->pf, c->lp, c->d_opsf, nullptr, c->d_rvol32, c->d_trace32, w, c->d_hi32[0], c->d_lo32[0],
                    nullptr, s);
     cudaMemsetAsync(c->d_dd32[0], 0, c->n32 * sizeof(float), s);
   }
@@ -918,7 +936,8 @@ extern "C" int dg_kernel_costs(const dg_ctx *c, double *flops, double *bytes, in
   // one-node-per-thread inviscid kernels, the state and volume parts as padded 8-word node records.
   const bool f64 = c->prec == DG_FP64;
   const double nt = f64 ? c->ks.nt : TRW32;
-  const double nw = f64 || visc || c->lines ? 7 : SW32;
+  const auto words = [&](int steps) { return f64 || visc || runs_lines(c, steps) ? 7.0 : (double)SW32; };
+  const double nw = words(GRAPH_UNROLL), n1 = words(1);
   const double word = f64 ? 8.0 : 4.0;
   if (!f64) fv += 3 * 2 * d * P1;  // compression term of the reduced energy
   const double bv = word * (E * Np * (nw + nw) + E * NFK * nt);
@@ -930,8 +949,8 @@ extern "C" int dg_kernel_costs(const dg_ctx *c, double *flops, double *bytes, in
   // 3 FP64 operations per variable for the split) and last surface kernel (reads the step start's
   // hi and lo, writes the FP64 state hi + lo: 9 operations of the float-float sum and 2 for the
   // sum per variable)
-  const double b3 = 8.0 * NV * E * Np + 4.0 * (E * Np * 3 * nw + E * NFK * nt);
-  const double b4 = 4.0 * (E * NFK * nt * 2 + E * Np * 4 * nw) + 8.0 * NV * E * Np;
+  const double b3 = 8.0 * NV * E * Np + 4.0 * (E * Np * 3 * n1 + E * NFK * nt);
+  const double b4 = 4.0 * (E * NFK * nt * 2 + E * Np * 4 * n1) + 8.0 * NV * E * Np;
   const int nk = std::min(nmax, c->prec == DG_FP64 ? 2 : 5);
   const double F[5] = {fv * E * Np, fs * E * Np, (fv + fs) * E * Np, (fv + 3 * NV) * E * Np, (fs + 11 * NV) * E * Np};
   const double Bb[5] = {bv, bs, bsv, b3, b4};

@@ -46,11 +46,13 @@
 // can write the FP64 state directly (hi + lo).  With the fused stage kernel
 // (k_surfvol32 below) n steps take 1 + 3n launches.
 //
-// These kernels give a node to a thread: the short chain for 1D problems and for
-// 2D meshes that do not fill the GPU, and the batches (dg_batch.cuh).  Larger
-// 2D meshes run the kernels of dg_lines32.cuh, one element line per thread
-// (use_lines32).
+// These kernels give a node to a thread: the short chain for 1D problems, for
+// 2D meshes that do not fill the GPU and for short calls, and the batches
+// (dg_batch.cuh).  Longer calls on larger 2D meshes run the kernels of
+// dg_lines32.cuh, one element line per thread (use_lines32).
 #pragma once
+
+#include <algorithm>
 
 #include "dg_common.cuh"
 #include "dg_kernels_fp64.cuh"
@@ -1064,7 +1066,10 @@ struct KernelSet32 {
   cudaError_t (*surfvol)(const Params &, const ParamsF &, const LineParams &, const float *opsf, int mode, float dt,
                          const StageIO &io, const float *rvol_in, const float *tr_in, float *rvol_out, float *tr_out,
                          cudaStream_t);
-  int wave_tiles;  // line kernels: tiles that the GPU holds at once (stage kernel); others: 0
+  // Elements (line kernels: tiles) that the GPU holds at once: of the stage kernel, and of the kernels at
+  // the FP64 ends of a call.
+  int (*resident_stage)();
+  int (*resident_ends)();
 };
 
 // A grid that the device holds at once is launched as a programmatic dependent
@@ -1120,8 +1125,14 @@ cudaError_t launch_surfvol32(const Params &prm, const ParamsF &pf, const LinePar
 
 template <int P, int DIM, bool VISC, bool ST>
 KernelSet32 make_set32() {
+  using G = Geom<P, DIM, VISC, ST>;
   return KernelSet32{&launch_volume32<P, DIM, VISC, ST>, &launch_surface32<P, DIM, VISC, ST>,
-                     &launch_surfvol32<P, DIM, VISC, ST>, 0};
+                     &launch_surfvol32<P, DIM, VISC, ST>,
+                     [] { return G::EPB * resident_blocks(k_surfvol32<P, DIM, VISC, ST, true>, G::THREADS); },
+                     [] {
+                       return G::EPB * std::min(resident_blocks(k_volume32<P, DIM, VISC, ST, true>, G::THREADS),
+                                                resident_blocks(k_surface32<P, DIM, VISC, ST, true>, G::THREADS));
+                     }};
 }
 
 template <int P>

@@ -19,7 +19,7 @@
 // viscous, surface tension: 780 instead of 1,560; no index arithmetic or divisions per face node, no
 // shared load per term), which is what bounds those on grids of many waves, but a thread's chain is
 // P + 1 times as long and a warp holds four to six times the nodes, so a mesh that does not fill the
-// GPU is left to the one-node-per-thread kernels (use_lines32).
+// GPU, and a call too short for its ends, is left to the one-node-per-thread kernels (use_lines32).
 // Measured, 10 steps of a viscous Rayleigh-Taylor problem with surface tension, 256 x 256, p = 4: 3082 us one
 // node per thread, 2795 here.  What bounds them is instruction issue with exposed load latency, at 12 warps
 // an SM.
@@ -131,21 +131,34 @@ inline int line_tiles(int P1, int E) { return (E + 32 / P1 - 1) / (32 / P1); }
 inline size_t line_node_floats(int P1, int E) { return (size_t)line_tiles(P1, E) * NV * P1 * 32; }
 inline size_t line_trace_floats(int P1, int E) { return (size_t)line_tiles(P1, E) * 4 * 3 * 32 * 4; }
 
-// Whether a single problem runs the line kernels: where a warp of them has enough others on its SM, and
-// the grid does not end in a thin last wave.  Below the first limit the longer chain of a line thread is
-// not hidden; a wave of line warps holds so many nodes that one just begun costs most of a full one.
-// wave: tiles that the GPU holds at once (stage kernel); full: viscous stress or surface tension.
-// Microseconds a step, one node / one line per thread, by line warps per SM (wave: 12; p = 5 full 8):
-//   p = 1        1.7: 14.8 / 11.3    6.7: 18.8 / 16.4   17.3: 45.9 / 33.5
-//   p = 2        2.7: 16.7 / 17.4    6.1: 28.6 / 20.9   16.8: 53.3 / 44.1   26.3: 85.3 / 61.5
-//   p = 2 full   2.7: 30.5 / 22.1   10.8: 51.5 / 29.0   16.4: 65.5 / 50.5
-//   p = 3        5.3: 25.8 / 23.1   11.5: 41.4 / 31.0   14.8: 47.1 / 50.3   16.1: 54.6 / 51.8   25.2: 88.9 / 79.7
-//   p = 3 full   7.6: 33.7 / 29.8   11.5: 41.1 / 34.0   14.8: 52.3 / 57.2   21.1: 71.3 / 65.9   25.2: 87.8 / 87.4
-//   p = 4        7.0: 32.7 / 27.9   11.4: 45.6 / 35.8   13.8: 54.1 / 53.8   18.0: 71.7 / 63.3   24.7: 100 / 90
-//   p = 4 full   7.0: 39.4 / 32.5   11.4: 53.5 / 41.4   13.8: 64.0 / 64.2   21.5: 97.6 / 81.7
-//   p = 5        5.4: 32.2 / 32.3   10.7: 52.3 / 46.3   15.3: 75.5 / 77.6   17.1: 87.3 / 82.5   21.6: 114 / 94
-//   p = 5 full   5.4: 37.0 / 35.1    7.8: 45.1 / 38.5   13.2: 73.8 / 76.5   15.3: 83.4 / 79.8   25.8: 144 / 156   33.7: 184 / 193
-inline bool use_lines32(int P1, bool full, int E, int wave) {
+// Which calls of a single problem run the line kernels: dg_rhs, and captured sequences of at least `steps`
+// steps (0: none).
+//
+// A thread's chain is P + 1 times as long here and a warp holds as many times the nodes, so the line kernels
+// need enough warps on every SM, and they lose where the one-node kernels' grid still fits on the GPU at once
+// (their time jumps by half when it no longer does) and where their own grid ends in a thin second wave.  The
+// kernels at the FP64 ends of a call stage the state through shared memory, at fewer warps per SM: they cost
+// what the stages between them win back only over several steps, and a right-hand side, which is nothing but
+// ends, pays while they fit on the GPU at once (inviscid up to p = 4: a little longer).  Times on one line per thread over times on one node per
+// thread, periodic in x, at w line warps per SM (right-hand side, sequences of 1, 2, 4 and 8 steps):
+//   p = 1        w 1.5: 1.13 1.13 1.15 1.05 0.89    2.6: 1.01 1.25 1.07 0.90 0.77    4.1: 0.69 1.00 0.89 0.81 0.75
+//   p = 1 visc.  w 1.5: 1.16 0.83 0.95 0.87 0.84    2.1: 0.80 0.90 0.86 0.81 0.72    26.9: 0.86 0.80 0.73 0.68 0.65
+//   p = 2        w 5.6: 0.84 1.11 1.13 1.11 1.08    6.1: 0.76 0.85 0.78 0.74 0.71   (one node: all resident up to 5.6)
+//   p = 2 visc.  w 1.8: 1.07 1.30 1.21 1.08 0.86    3.4: 0.95 1.06 0.93 0.76 0.65    5.6: 0.91 0.97 0.78 0.67 0.62
+//   p = 3        w 4.8: 1.22 1.48 1.50 1.42 1.40    5.3: 0.88 1.00 0.97 0.92 0.89   12.6: 1.00 1.15 1.21 1.13 1.09
+//                w 17.1: 1.11 1.12 1.04 0.97 0.93   30.3: 1.00 0.97 0.95 0.89 0.87
+//   p = 3 visc.  w 7.0: 0.90 1.20 1.23 1.26 1.24    8.2: 0.85 1.00 0.95 0.92 0.89   25.5: 1.25 1.15 1.09 1.03 1.00
+//   p = 4        w 5.7: 0.93 1.14 1.15 1.12 1.11    7.0: 0.90 1.00 0.94 0.89 0.86   18.0: 1.09 1.06 0.99 0.93 0.89
+//   p = 4 tens.  w 8.5: 0.91 0.91 0.93 0.88 0.85   11.9: 0.85 0.89 0.86 0.80 0.76   18.0: 1.09 1.08 1.02 0.95 0.92
+//   p = 4 visc.  w 8.5: 1.13 1.00 0.95 0.88 0.84   18.0: 1.28 1.10 1.05 0.96 0.92   71.9: 1.19 1.07 1.00 0.93 0.90
+//   p = 5        w 7.6: 0.80 0.98 1.00 0.96 0.94    8.4: 1.15 1.15 1.15 1.01 0.93   27.3: 1.27 1.15 1.10 1.01 0.97
+//   p = 5 full   w 6.8: 0.83 0.96 0.99 0.92 0.89    8.4: 1.47 1.39 1.47 1.30 1.22   33.7: 1.29 1.25 1.16 1.07 1.02
+// (surface tension alone as inviscid, except at p = 5, where any term takes the registers.)
+struct LineUse {
+  bool rhs;
+  int steps;
+};
+inline LineUse use_lines32(int P1, bool viscous, bool tension, int E, const KernelSet32 &one, const KernelSet32 &line) {
   static const int sms = [] {
     int dev = 0, n = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -153,13 +166,31 @@ inline bool use_lines32(int P1, bool full, int E, int wave) {
       n = 152;
     return n;
   }();
-  const int tiles = line_tiles(P1, E);
-  if (2 * tiles < (P1 > 3 ? 10 : P1 == 3 && !full ? 8 : 3) * sms) return false;
-  if (P1 <= 3 || tiles <= wave) return true;
-  if (P1 == 6 && full) return false;
+  const long long tiles = line_tiles(P1, E), w = 10 * tiles / sms;  // line warps per SM, in tenths
+  if (P1 == 2) {
+    if (w < 15) return {false, 0};
+    return {w >= (viscous ? 20 : 28), viscous || w >= 40 ? 1 : w >= 30 ? 2 : w >= 20 ? 3 : 5};
+  }
+  if (P1 == 3) {
+    if (w < 15) return {false, 0};
+    const bool rhs = w >= 24;
+    if (!viscous) return {rhs, E > one.resident_stage() ? 1 : 0};
+    return {rhs, w >= 50 ? 1 : w >= 30 ? 2 : w >= 21 ? 4 : 6};
+  }
+  if (w < 50) return {false, 0};
+  const bool full5 = P1 == 6 && (viscous || tension), few5 = P1 == 6 && w < 60;
+  const long long wave = line.resident_stage();
+  LineUse u{!few5 && tiles <= (viscous || P1 == 6 ? line.resident_ends() : wave), 0};
+  if (E <= one.resident_stage()) return u;
+  if (tiles <= wave) {
+    u.steps = P1 < 6 || (full5 && !few5) ? 1 : few5 && !full5 ? 0 : 5;
+    return u;
+  }
   // percent of the second wave that has to be there; in later ones it matters no more
-  const int least = P1 == 4 && full ? 60 : 35;
-  return tiles > 2LL * wave || 100LL * (tiles - wave) >= (long long)least * wave;
+  const int least = P1 == 4 && (viscous || tension) ? 60 : 35;
+  if (full5 || (tiles <= 2 * wave && 100 * (tiles - wave) < least * wave)) return u;
+  u.steps = P1 == 6 || (P1 == 4 && viscous) ? 5 : viscous ? 3 : 2;
+  return u;
 }
 
 template <int P1>
@@ -1096,7 +1127,11 @@ template <int P, bool VISC, bool ST>
 KernelSet32 make_lines32() {
   return KernelSet32{&launch_volume32_lines<P, VISC, ST>, &launch_surface32_lines<P, VISC, ST>,
                      &launch_surfvol32_lines<P, VISC, ST>,
-                     WPB32 * resident_blocks(k_surfvol32_lines<P, VISC, ST, true>, 32 * WPB32)};
+                     [] { return WPB32 * resident_blocks(k_surfvol32_lines<P, VISC, ST, true>, 32 * WPB32); },
+                     [] {
+                       return WPB32 * std::min(resident_blocks(k_volume32_lines<P, VISC, ST, true>, 32 * WPB32),
+                                               resident_blocks(k_surface32_lines<P, VISC, true>, 32 * WPB32));
+                     }};
 }
 
 // Line kernels of order P (2D).
