@@ -60,7 +60,7 @@ struct LineParams {
   float p_bc[4];
   float eta_x, eta_y;
   float C2, dC, g2, dg, Bp;
-  float rho01, rho02, drho0, mu2, dmu, sigma, gx, gy, Gamma, eps;
+  float rho01, rho02, drho0, mu1, mu2, sigma, gx, gy, Gamma, eps;
   int gravity, check_finite;
   double C2d, dCd;
   unsigned *status;
@@ -90,8 +90,8 @@ __host__ inline LineParams line_params(const Params &p, int P1, const float *ops
   f.rho01 = (float)p.rho01;
   f.rho02 = (float)p.rho02;
   f.drho0 = (float)p.drho0;
+  f.mu1 = (float)p.mu1;
   f.mu2 = (float)p.mu2;
-  f.dmu = (float)p.mu1 - (float)p.mu2;
   f.sigma = (float)p.sigma;
   f.gx = (float)p.gx;
   f.gy = (float)p.gy;
@@ -105,6 +105,12 @@ __host__ inline LineParams line_params(const Params &p, int P1, const float *ops
   f.opsf = d_opsf;
   for (int k = 0; k < P1 * P1; ++k) f.D[k] = opsf[k];
   return f;
+}
+
+// phi_1 mu_1 + phi_2 mu_2: either phase's own viscosity where the other is absent, whatever their ratio
+// (mu_2 + phi (mu_1 - mu_2) loses the smaller one in the difference's rounding).
+__device__ __forceinline__ float mixture_mu(const LineParams &pf, float phi) {
+  return pf.mu1 * phi + pf.mu2 * (1.f - phi);
 }
 
 // Geometry.  NL lines (threads) per element, EPW elements per warp.  Shared memory: a line is padded
@@ -429,7 +435,7 @@ __device__ __forceinline__ void face_flux32(const LineParams &pf, const float *t
     }
   }
   if (VISC) {
-    const float mm = fmaf(pf.dmu, tm[PHI], pf.mu2), mp = fmaf(pf.dmu, tp[PHI], pf.mu2), mua = 0.5f * (mp + mm);
+    const float mua = 0.5f * (mixture_mu(pf, tp[PHI]) + mixture_mu(pf, tm[PHI]));
     const float tmx = tm[LT_TX] * sg, tmy = tm[LT_TY] * sg, tpx = tp[LT_TX] * sg, tpy = tp[LT_TY] * sg;
     // tau^ . m - tau- . m
     S[RU] += wf * (0.5f * (tpx - tmx) + eta * mua * (p.u - m.u));
@@ -551,7 +557,7 @@ __device__ __forceinline__ void vol32_line(const LineParams &pf, float *sm, cons
     nc[i] = u[i] * gpx[i] + v[i] * gpy[i];
     R[PSI][i] = -(u[i] * gsx[i] + v[i] * gsy[i]);
     if (VISC) {
-      const float mu = fmaf(pf.dmu, q[PHI][i], pf.mu2);
+      const float mu = mixture_mu(pf, q[PHI][i]);
       const float div3 = (gux[i] + gvy[i]) * (1.f / 3.f);
       txx[i] = 2.f * mu * (gux[i] - div3);
       tyy[i] = 2.f * mu * (gvy[i] - div3);

@@ -11,7 +11,7 @@ import pytest
 
 from paper_2306_05002_gb300 import workloads as W
 from tests.helpers import problem
-from tests.test_gpu_fp32bulk import _l2, _rhs32
+from tests.test_gpu_fp32bulk import TOL32, _l2, _rhs32, _storage_bound
 
 pytestmark = pytest.mark.gpu
 TERMS = {"none": (False, False), "tension": (False, True), "viscous": (True, False), "both": (True, True)}
@@ -150,3 +150,24 @@ def test_failures_in_the_ragged_tile(dg, p, warps):
     s.dg_step(torch.from_numpy(wl.w.copy()).cuda(), wl.dt, 8)
     assert s.dg_status_read() == 0
     s.close()
+
+
+@pytest.mark.parametrize("p,warps", [(1, 5.2), (2, 7.0), (3, 9.0), (4, 6.0), (5, 6.6)])
+@pytest.mark.parametrize("phase", [0, 1])
+def test_viscosity_of_a_pure_phase(orc, dg, p, warps, phase):
+    """One phase alone, of 1e-8 times the other's viscosity: the mixture's is its own.  The rows that
+    viscosity enters, momentum and energy (those of the absent phase are zero to the oracle's rounding)."""
+    import torch
+    n = _side(p, warps)
+    wl = W.Workload(name="pure", dim=2, nx=n, ny=n, p=p, viscous=True, mu=(1e5, 1e13) if phase == 0 else (1e13, 1e5))
+    x, y = W.node_coords(wl)
+    wl.w = W.conserved(wl, np.full(wl.N, 1.0 - phase), 0.2 * np.sin(2 * np.pi * y), 1e5,
+                       0.3 * np.sin(2 * np.pi * y), 0.2 * np.cos(2 * np.pi * x))
+    assert _routes(dg, wl)[0] == 1
+    L_ref, S = orc.rhs(problem(orc, wl), wl.w, want_scale=True)
+    s = dg.Solver(wl, precision="fp32bulk")
+    L = s.dg_rhs(torch.from_numpy(wl.w.copy()).cuda()).cpu().numpy()
+    s.close()
+    extra = _storage_bound(orc, wl, wl.w)
+    for v in (4, 5, 6):
+        assert np.abs(L[v] - L_ref[v]).max() <= TOL32 * S[v].max() + extra.get(v, 0.0), v
