@@ -209,10 +209,11 @@ dg_status dg_status_read(dg_ctx *ctx, void *stream);
    The normal build compiles the checks out. */
 int dg_check_build(long long *failures);
 
-/* Self-test of the bounds-checked build: runs the FP64 volume kernel of a
-   small problem with a node count one short of the mesh's (every array keeps
-   its true size, so no access leaves its allocation) and returns 1 when the
-   last node's index check caught it (latched and skipped), 0 when it did not,
+/* Self-test of the bounds-checked build: runs the FP64 volume kernel and the
+   FP32-bulk line kernels of a small problem with a node count one short of the
+   mesh's (every array keeps its true size, so no access leaves its allocation)
+   and returns 1 when every kernel's check caught it (latched and skipped), 0
+   when one did not,
    DG_ERR_CUDA on a CUDA failure and DG_ERR_UNSUPPORTED in the normal build.
    Synchronises stream; the planted failure is not counted by dg_check_build. */
 int dg_check_selftest(void *stream);

@@ -519,10 +519,47 @@ extern "C" void dg_destroy(dg_ctx *c) {
   free_ctx(c);
 }
 
-// Self-test of the bounds-checked build: the FP64 volume kernel of a 2 x 2, p = 2 periodic problem
-// runs with a node count one short of the mesh's.  Every array keeps its true size, so no access
-// leaves its allocation (the field offsets v (N - 1) + n stay below 7 N); only the last node's
-// index fails its check, which must latch STATUS_BOUNDS and skip that node.
+// Self-test of the bounds-checked build: the FP64 volume kernel and the FP32-bulk line kernels of a
+// 2 x 2, p = 2 periodic problem run with a node count one short of the mesh's.  Every array keeps its
+// true size, so no access leaves its allocation (the field offsets v (N - 1) + n stay below 7 N, and
+// the line kernels' arrays are indexed by tile); only the last node's index fails its check, which
+// must latch STATUS_BOUNDS in each kernel and skip that node.
+#ifdef DG_CHECK
+static bool caught(dg_ctx *c, cudaStream_t s, cudaError_t launched, cudaError_t *e) {
+  unsigned word = 0;
+  if (*e == cudaSuccess) *e = launched;
+  if (*e == cudaSuccess) *e = cudaMemcpyAsync(&word, c->d_status, sizeof(unsigned), cudaMemcpyDeviceToHost, s);
+  if (*e == cudaSuccess) *e = cudaMemsetAsync(c->d_status, 0, sizeof(unsigned), s);  // planted: not a failure
+  if (*e == cudaSuccess) *e = cudaStreamSynchronize(s);
+  return *e == cudaSuccess && (word & STATUS_BOUNDS);
+}
+
+// The line kernels of c's mesh with the parameters q, on node arrays of their own.
+static bool lines_caught(dg_ctx *c, const Params &q, cudaStream_t s, cudaError_t *e) {
+  KernelSet32 kl;
+  lines_fp32(c->p, false, false, &kl);
+  const std::vector<double> ops = build_ops(c->dim, c->p, c->hx, c->hy);
+  const std::vector<float> opsf(ops.begin(), ops.end());
+  const size_t nn = line_node_floats(c->P1, c->E), nt = line_trace_floats(c->P1, c->E);  // multiples of 4
+  float *buf = nullptr;
+  *e = cudaMalloc(&buf, (5 * nn + 2 * nt + opsf.size()) * sizeof(float));
+  if (*e != cudaSuccess) return false;
+  float *hi = buf, *d0 = hi + nn, *d1 = d0 + nn, *rv = d1 + nn, *rv2 = rv + nn, *tr = rv2 + nn, *tr2 = tr + nt,
+        *ops_dev = tr2 + nt;
+  *e = cudaMemsetAsync(buf, 0, (5 * nn + 2 * nt) * sizeof(float), s);
+  if (*e == cudaSuccess)
+    *e = cudaMemcpyAsync(ops_dev, opsf.data(), opsf.size() * sizeof(float), cudaMemcpyHostToDevice, s);
+  const LineParams lp = line_params(q, c->P1, opsf.data(), ops_dev);
+  const StageIO io{hi, nullptr, d0, d1, nullptr, nullptr, nullptr, nullptr, nullptr};
+  bool ok = true;
+  ok &= caught(c, s, kl.volume(q, c->pf, lp, ops_dev, hi, rv, tr, nullptr, nullptr, nullptr, nullptr, s), e);
+  ok &= caught(c, s, kl.surfvol(q, c->pf, lp, ops_dev, MODE_S2, 0.f, io, rv, tr, rv2, tr2, s), e);
+  ok &= caught(c, s, kl.surface(q, c->pf, lp, ops_dev, MODE_S2, 0.f, io, rv, tr, s), e);
+  cudaFree(buf);
+  return ok;
+}
+#endif
+
 extern "C" int dg_check_selftest(void *stream) {
 #ifndef DG_CHECK
   (void)stream;
@@ -552,16 +589,13 @@ extern "C" int dg_check_selftest(void *stream) {
   Params q = c->prm;
   q.N -= 1;
   q.check_finite = 0;
-  unsigned word = 0;
   cudaError_t e = cudaMemcpyAsync(c->d_w1, h.data(), c->len * sizeof(double), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->d_status, 0, sizeof(unsigned), s);
-  if (e == cudaSuccess) e = c->ks.volume(q, c->d_w1, c->d_rvol, c->d_trace, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&word, c->d_status, sizeof(unsigned), cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(c->d_status, 0, sizeof(unsigned), s);  // planted: not a failure
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  bool ok = caught(c, s, e == cudaSuccess ? c->ks.volume(q, c->d_w1, c->d_rvol, c->d_trace, s) : e, &e);
+  if (e == cudaSuccess) ok &= lines_caught(c, q, s, &e);
   dg_destroy(c);
   if (e != cudaSuccess) return DG_ERR_CUDA;
-  return (word & STATUS_BOUNDS) ? 1 : 0;
+  return ok ? 1 : 0;
 #endif
 }
 

@@ -913,6 +913,15 @@ __host__ __device__ constexpr int line_smem(int fields) {
   return ((a > b ? a : b) + 3) / 4 * 4;
 }
 
+// Whether a tile's last node lies below the node count, and with it the tile's slots in the node arrays
+// (the bounds-checked build; else constant true).  The whole warp agrees.
+template <int P>
+__device__ __forceinline__ bool tile_in_bounds(const LineParams &pf, int tile) {
+  using G = LineGeom<P>;
+  const long long end = (long long)(tile + 1) * G::EPW;
+  return in_bounds(pf.status, (end < pf.E ? end : pf.E) * G::NP - 1, pf.N);
+}
+
 // Bodies of the three kernels for one tile (tiles past the mesh are skipped by the whole warp).
 template <int P, bool VISC, bool ST, bool PDL>
 __device__ __forceinline__ void volume32_tile(const LineParams &pf, float *sm, int tile, const float *__restrict__ w,
@@ -920,7 +929,7 @@ __device__ __forceinline__ void volume32_tile(const LineParams &pf, float *sm, i
                                               const double *__restrict__ w64, float *__restrict__ w32out,
                                               float *__restrict__ lo_out, double *__restrict__ w64copy) {
   using G = LineGeom<P>;
-  if (tile * G::EPW >= pf.E) return;
+  if (tile * G::EPW >= pf.E || !tile_in_bounds<P>(pf, tile)) return;
   const LinePlace<P> pl(pf.E, tile);
   float q[NV][G::P1];
   if (w64) load_state64<P, PDL>(pf, sm, pl, w64, w32out, lo_out, w64copy, q);
@@ -933,7 +942,7 @@ __device__ __forceinline__ void surfvol32_tile(const LineParams &pf, float *sm, 
                                                const StageIO &io, const float *__restrict__ rvol_in,
                                                const float4 *__restrict__ tr_in, float *__restrict__ rvol_out,
                                                float4 *__restrict__ tr_out) {
-  if (tile * LineGeom<P>::EPW >= pf.E) return;
+  if (tile * LineGeom<P>::EPW >= pf.E || !tile_in_bounds<P>(pf, tile)) return;
   const LinePlace<P> pl(pf.E, tile);
   float L[NV][P + 1];
   surf32_line<P, VISC, PDL>(pf, sm, pl, rvol_in, tr_in, L);
@@ -949,7 +958,7 @@ __device__ __forceinline__ void surface32_tile(const LineParams &pf, float *sm, 
                                                const float4 *__restrict__ tr) {
   using G = LineGeom<P>;
   constexpr int P1 = G::P1;
-  if (tile * G::EPW >= pf.E) return;
+  if (tile * G::EPW >= pf.E || !tile_in_bounds<P>(pf, tile)) return;
   const LinePlace<P> pl(pf.E, tile);
   float L[NV][P1];
   surf32_line<P, VISC, PDL>(pf, sm, pl, rvol, tr, L);
