@@ -277,11 +277,9 @@ k_kin_stage(const KinParams kp, int epb, int mode, int ic, bool last, double *w0
   const int le_raw = threadIdx.x / NP, a = threadIdx.x % NP;
   const bool lane = le_raw < epb;
   const int le = lane ? le_raw : epb - 1, e0 = blockIdx.x * epb + le;
-  // (idle lanes take an element of their own block: another's nodes may be being written)
-  const int ec = e0 < kp.E ? e0 : kp.E - 1;
-  const bool ok = in_bounds(kp.status, (long long)ec * NP + a, N);
-  const bool act = lane && e0 < kp.E && ok;
-  const int e = ok ? ec : 0;
+  const bool act = lane && e0 < kp.E && in_bounds(kp.status, (long long)e0 * NP + a, N);
+  // (idle lanes take their own block's first element: another block's nodes may be being written)
+  const int e = act ? e0 : blockIdx.x * epb;
   const long n = (long)e * NP + a;
   double r[2], base[2] = {0.0, 0.0};
 #pragma unroll

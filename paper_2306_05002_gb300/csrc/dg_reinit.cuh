@@ -177,14 +177,16 @@ k_ri_stage(const ReinitParams rp, int epb, int mode, double dtau, bool last, dou
   const int le_raw = threadIdx.x / NP, a = threadIdx.x % NP;
   const bool lane = le_raw < epb;
   const int le = lane ? le_raw : epb - 1, e0 = blockIdx.x * epb + le;
-  // (idle lanes take an element of their own block: another's nodes may be being written)
-  const int ec = e0 < rp.E ? e0 : rp.E - 1;
-  const bool ok = in_bounds(rp.status, (long long)ec * NP + a, rp.N);
-  const bool act = lane && e0 < rp.E && ok;
-  const int e = ok ? ec : 0;
+  const bool act = lane && e0 < rp.E && in_bounds(rp.status, (long long)e0 * NP + a, rp.N);
+  const int e = act ? e0 : 0;
   const long n = (long)e * NP + a;
-  const double p0 = __ldca(psi + n), pw = mode == MODE_S1 ? p0 : __ldca(ws + n);
-  double r = __ldca(rvol + n);
+  // (idle lanes read no node: another block may be writing it)
+  double p0 = 0.0, pw = 0.0, r = 0.0;
+  if (act) {
+    p0 = __ldca(psi + n);
+    r = __ldca(rvol + n);
+    pw = mode == MODE_S1 ? p0 : __ldca(ws + n);
+  }
 
   for (int g = threadIdx.x; g < fs; g += blockDim.x) {
     const int fe = blockIdx.x * epb + g / NFK, t = g % NFK;
