@@ -273,7 +273,9 @@ struct dg_ctx {
   int tri_grid = 0, tri_epb = 1;
   double *d_kacc = nullptr, *d_kwsA = nullptr, *d_kwsB = nullptr;
   double *d_kt = nullptr, *d_kxi = nullptr, *d_ktv = nullptr;
-  double *d_krvol = nullptr, *d_ktr = nullptr;  // rectangles: volume part, two buffers of face traces
+  // rectangles: volume part, two buffers of face traces (ktr2; one where two do not fit)
+  double *d_krvol = nullptr, *d_ktr = nullptr;
+  bool ktr2 = true;
   // level-set re-initialisation workspace (dg_reinit), allocated on first use
   double *d_riS = nullptr, *d_ri1 = nullptr, *d_rirvol = nullptr, *d_ritr = nullptr;
   double *d_part = nullptr, *d_diag = nullptr;
@@ -313,6 +315,18 @@ static dg_status fail(dg_ctx *c, dg_status s, const std::string &msg) {
   if (c) c->err = msg;
   else g_create_error = msg;
   return s;
+}
+
+// Face traces for stage kernels that read one buffer and write the other, or, where device memory does
+// not hold two (a state of N doubles per field has up to 2 N face nodes), one buffer: then every stage
+// is a volume and a stage launch.
+static cudaError_t trace_buffers(double **p, size_t len, bool *two) {
+  *two = true;
+  cudaError_t e = cudaMalloc(p, 2 * len * sizeof(double));
+  if (e != cudaErrorMemoryAllocation) return e;
+  cudaGetLastError();
+  *two = false;
+  return cudaMalloc(p, len * sizeof(double));
 }
 
 static dg_status cuda_fail(dg_ctx *c, cudaError_t e, const char *what) {
@@ -1392,7 +1406,6 @@ extern "C" dg_status dg_kin_create(const dg_mesh *mesh, int p, double Gamma, dou
     if (e == cudaSuccess) e = cudaMalloc(&c->d_kwsB, sb);
   } else {
     if (e == cudaSuccess) e = cudaMalloc(&c->d_krvol, sb);
-    if (e == cudaSuccess) e = cudaMalloc(&c->d_ktr, (size_t)2 * KIN_NT * c->E * c->NFK * sizeof(double));
   }
   // the velocity's spatial factor at every node (rectangles) or quadrature point (triangles)
   const size_t vrows = tri ? (size_t)c->E * c->tk.points : (size_t)c->N;
@@ -1412,6 +1425,10 @@ extern "C" dg_status dg_kin_create(const dg_mesh *mesh, int p, double Gamma, dou
   if (e == cudaSuccess) e = cudaMalloc(&c->d_ops, ops.size() * sizeof(double));
   if (e == cudaSuccess) e = cudaMalloc(&c->d_status, sizeof(unsigned));
   if (e == cudaSuccess) e = cudaMemcpy(c->d_ops, ops.data(), ops.size() * sizeof(double), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess && !tri) {
+    e = trace_buffers(&c->d_ktr, (size_t)KIN_NT * c->E * c->NFK, &c->ktr2);
+    if (e == cudaSuccess && !c->ktr2) e = cudaMalloc(&c->d_kwsA, sb);  // the stage state
+  }
   if (e == cudaSuccess) e = cudaMemcpy(c->d_kxi, xi.data(), xi.size() * sizeof(double), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemset(c->d_kt, 0, KT_SIZE * sizeof(double));
   if (e == cudaSuccess) e = cudaMemset(c->d_status, 0, sizeof(unsigned));
@@ -1502,21 +1519,28 @@ extern "C" dg_status dg_kin_rhs(dg_ctx *c, const double *w, double t, double *L,
 // `steps` classical RK4 steps of the captured sequence.  The kernels read the step size and the stage
 // times' velocity factors from device memory (c->d_kt), stage st of step k at index 4 k + st.
 // Rectangles: the volume part of the first stage, then one launch per stage that leaves the volume
-// part and the traces of the next one; the trace buffers alternate.  Triangles: stage inputs
-// w -> A -> B -> A, the last stage writes w in place.
+// part and the traces of the next one; the trace buffers alternate (one buffer: a volume launch before
+// every stage, on the stage state A).  Triangles: stage inputs w -> A -> B -> A, the last stage writes w
+// in place.
 static dg_status enqueue_kin_steps(dg_ctx *c, double *w, int steps, cudaStream_t s) {
   const int mode[4] = {KIN_K1, KIN_K2, KIN_K3, KIN_K4};
   double *A = c->d_kwsA, *B = c->d_kwsB;
   const double *in[4] = {w, A, B, A};
   double *out[4] = {A, B, A, w};
   const size_t half = (size_t)KIN_NT * c->E * c->NFK;
-  cudaError_t e = c->tri ? cudaSuccess : c->kk.volume(c->kp, 0, w, c->d_krvol, c->d_ktr, s);
+  cudaError_t e = c->tri || !c->ktr2 ? cudaSuccess : c->kk.volume(c->kp, 0, w, c->d_krvol, c->d_ktr, s);
   for (int q = 0; q < 4 * steps && e == cudaSuccess; ++q) {
-    if (c->tri)
+    if (c->tri) {
       e = c->tk.stage(c->kp, mode[q & 3], q, in[q & 3], w, c->d_kacc, out[q & 3], c->tri_epb, c->tri_grid, s);
-    else
+    } else if (!c->ktr2) {
+      const bool end = (q & 3) == 3;
+      e = c->kk.volume(c->kp, q, (q & 3) ? A : w, c->d_krvol, c->d_ktr, s);
+      if (e == cudaSuccess)
+        e = c->kk.stage(c->kp, mode[q & 3], q, true, w, c->d_kacc, c->d_krvol, c->d_ktr, nullptr, end ? w : A, s);
+    } else {
       e = c->kk.stage(c->kp, mode[q & 3], q, q == 4 * steps - 1, w, c->d_kacc, c->d_krvol, c->d_ktr + (q & 1) * half,
                       c->d_ktr + (~q & 1) * half, w, s);
+    }
   }
   return e == cudaSuccess ? DG_OK : cuda_fail(c, e, "dg_kin_step: launch");
 }

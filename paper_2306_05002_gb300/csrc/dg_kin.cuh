@@ -251,7 +251,8 @@ k_kin_volume(const KinParams kp, int epb, int ic, const double *__restrict__ w, 
 //   K4: r = w0 + dt/6 (acc + L), written to w0 (each node by the thread that read it);
 // then, unless last, the volume part of the next stage on r (time factor kt[KT_C + ic + 1]; stage
 // index ic of the captured sequence), into rvol (the node's own value was read before) and the
-// other trace buffer, which neighbouring blocks of this launch do not read.
+// other trace buffer, which neighbouring blocks of this launch do not read.  r itself is written (out)
+// by K4, and by every stage that is the last before a volume launch.
 // Bound by the FP64 pipe: about 65 operations per node at p = 3, where a stage that evaluated the
 // neighbours' gradients and normals at every face node itself took about 150 (64 x 64, p = 3: an RK4
 // step 85 -> 44 us).
@@ -353,7 +354,7 @@ k_kin_stage(const KinParams kp, int epb, int mode, int ic, bool last, double *w0
   }
   if (act) {
     if (kp.check_finite && !(finite64(r[0]) && finite64(r[1]))) atomicOr(kp.status, STATUS_NONFINITE);
-    if (mode == KIN_RHS || mode == KIN_K4) {
+    if (mode == KIN_RHS || mode == KIN_K4 || last) {
       out[n] = r[0];
       out[N + n] = r[1];
     }
