@@ -278,6 +278,7 @@ struct dg_ctx {
   bool ktr2 = true;
   // level-set re-initialisation workspace (dg_reinit), allocated on first use
   double *d_riS = nullptr, *d_ri1 = nullptr, *d_rirvol = nullptr, *d_ritr = nullptr;
+  bool ritr2 = true;  // two buffers of face traces (trace_buffers)
   double *d_part = nullptr, *d_diag = nullptr;
   unsigned *d_status = nullptr;
   int nparts = 0;
@@ -1626,11 +1627,11 @@ extern "C" dg_status dg_reinit(dg_ctx *c, double *w, int niter, double nu, doubl
   if (!(dtau > 0.0)) dtau = std::min(0.5 * h / q, 0.1 * h * h / (q * q * rp.nu));
   cudaError_t e = cudaSuccess;
   if (!c->d_riS) {
-    const size_t nb = (size_t)rp.N * sizeof(double), tb = (size_t)4 * rp.E * rk.nfk * sizeof(double);
+    const size_t nb = (size_t)rp.N * sizeof(double);
     double **bufs[] = {&c->d_riS, &c->d_ri1, &c->d_rirvol};
     for (double **b : bufs)
       if (e == cudaSuccess) e = cudaMalloc(b, nb);
-    if (e == cudaSuccess) e = cudaMalloc(&c->d_ritr, tb);
+    if (e == cudaSuccess) e = trace_buffers(&c->d_ritr, (size_t)2 * rp.E * rk.nfk, &c->ritr2);
     if (e != cudaSuccess) {
       for (double **b : {&c->d_riS, &c->d_ri1, &c->d_rirvol, &c->d_ritr}) {
         cudaFree(*b);
@@ -1644,14 +1645,19 @@ extern "C" dg_status dg_reinit(dg_ctx *c, double *w, int niter, double nu, doubl
   cudaStream_t s = (cudaStream_t)stream;
   double *psi = w + rp.N;
   e = rk.sign(rp, w, c->d_riS, s);
-  // one launch per stage after the first volume part; the two trace buffers alternate
+  // one launch per stage after the first volume part; the two trace buffers alternate (one buffer: a
+  // volume launch before every stage)
   const int mode[3] = {MODE_S1, MODE_S2, MODE_S3};
   const long long nst = 3LL * niter;
   const size_t half = (size_t)2 * rp.E * rk.nfk;
-  if (e == cudaSuccess && niter > 0) e = rk.volume(rp, psi, c->d_riS, c->d_rirvol, c->d_ritr, s);
-  for (long long q = 0; q < nst && e == cudaSuccess; ++q)
-    e = rk.stage(rp, mode[q % 3], dtau, q == nst - 1, psi, c->d_ri1, c->d_riS, c->d_rirvol, c->d_ritr + (q & 1) * half,
-                 c->d_ritr + (~q & 1) * half, s);
+  for (long long q = 0; q < nst && e == cudaSuccess; ++q) {
+    if (q == 0 || !c->ritr2) e = rk.volume(rp, q % 3 ? c->d_ri1 : psi, c->d_riS, c->d_rirvol, c->d_ritr, s);
+    if (e == cudaSuccess && c->ritr2)
+      e = rk.stage(rp, mode[q % 3], dtau, q == nst - 1, psi, c->d_ri1, c->d_riS, c->d_rirvol,
+                   c->d_ritr + (q & 1) * half, c->d_ritr + (~q & 1) * half, s);
+    else if (e == cudaSuccess)
+      e = rk.stage(rp, mode[q % 3], dtau, true, psi, c->d_ri1, c->d_riS, c->d_rirvol, c->d_ritr, nullptr, s);
+  }
   return e == cudaSuccess ? DG_OK : cuda_fail(c, e, "dg_reinit: launch");
 }
 

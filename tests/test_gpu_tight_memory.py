@@ -89,3 +89,22 @@ s.close()
 """)
     for k in ("rhs", "1", "8", "11"):
         assert np.array_equal(r["plain_" + k], r["tight_" + k]), k
+
+
+@pytest.mark.parametrize("dim,p", [(1, 3), (2, 1), (2, 4)])
+def test_reinitialisation_with_one_trace_buffer(dg, wrapped, tmp_path, dim, p):
+    n = 37 if dim == 2 else 301
+    nfk = 4 * n * n * (p + 1) if dim == 2 else 2 * n
+    size = 2 * 2 * nfk * 8  # two buffers of two fields per face node
+    make = f"W.drop_2d({n}, {p})" if dim == 2 else f"W.slab_1d({n}, {p})"
+    r = _both(wrapped, tmp_path, size, f"""
+wl = {make}
+s = dg.Solver(wl)
+w = torch.from_numpy(wl.w.copy()).cuda()
+for k in (1, 4):
+    s.dg_reinit(w, k)
+    out[tag + "_%d" % k] = w.cpu().numpy()
+s.close()
+""")
+    for k in ("1", "4"):
+        assert np.array_equal(r["plain_" + k], r["tight_" + k]), k
