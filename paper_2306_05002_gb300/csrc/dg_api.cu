@@ -478,16 +478,31 @@ extern "C" dg_status dg_create(const dg_mesh *mesh, int p, const dg_eos *eos, do
       c->lu = use_lines32(P1, o.viscous != 0, o.surface_tension != 0, c->E, c->ks32, c->ksl);
     // one padded record per node (inviscid kernels) and per face node, and room for the line kernels' tiles:
     // every call writes what it reads, so calls on either layout share the arrays
-    size_t n32 = (size_t)SW32 * c->N, t32 = (size_t)TRW32 * c->E * c->NFK;
-    if (c->lu.rhs || c->lu.steps) {
-      n32 = std::max(n32, line_node_floats(P1, c->E));
-      t32 = std::max(t32, line_trace_floats(P1, c->E));
+    const struct {
+      float **p;
+      bool trace;
+    } bufs[] = {{&c->d_hi32[0], false}, {&c->d_hi32[1], false}, {&c->d_lo32[0], false}, {&c->d_lo32[1], false},
+                {&c->d_dd32[0], false}, {&c->d_dd32[1], false}, {&c->d_rvol32, false},  {&c->d_trace32, true},
+                {&c->d_rvol32b, false}, {&c->d_trace32b, true}};
+    alloc32(&c->d_opsf, opsf.size());
+    for (;;) {
+      const bool lines = c->lu.rhs || c->lu.steps;
+      size_t n32 = (size_t)SW32 * c->N, t32 = (size_t)TRW32 * c->E * c->NFK;
+      if (lines) {
+        n32 = std::max(n32, line_node_floats(P1, c->E));
+        t32 = std::max(t32, line_trace_floats(P1, c->E));
+      }
+      c->n32 = n32;
+      for (const auto &b : bufs) alloc32(b.p, b.trace ? t32 : n32);
+      if (e != cudaErrorMemoryAllocation || !lines) break;
+      for (const auto &b : bufs) {  // the tiles' padding does not fit: one node per thread for every call
+        cudaFree(*b.p);
+        *b.p = nullptr;
+      }
+      cudaGetLastError();
+      c->lu = LineUse{false, 0};
+      e = cudaSuccess;
     }
-    c->n32 = n32;
-    alloc32(&c->d_opsf, opsf.size()) && alloc32(&c->d_hi32[0], n32) && alloc32(&c->d_hi32[1], n32) &&
-        alloc32(&c->d_lo32[0], n32) && alloc32(&c->d_lo32[1], n32) && alloc32(&c->d_dd32[0], n32) &&
-        alloc32(&c->d_dd32[1], n32) && alloc32(&c->d_rvol32, n32) && alloc32(&c->d_trace32, t32) &&
-        alloc32(&c->d_rvol32b, n32) && alloc32(&c->d_trace32b, t32);
   }
   if (e != cudaSuccess || (e = cudaMalloc(&c->d_ops, ops.size() * sizeof(double))) != cudaSuccess ||
       (f64 && ((e = cudaMalloc(&c->d_w1, sbytes)) != cudaSuccess || (e = cudaMalloc(&c->d_w2, sbytes)) != cudaSuccess ||

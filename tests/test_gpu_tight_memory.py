@@ -10,6 +10,10 @@ import sys
 import numpy as np
 import pytest
 
+from paper_2306_05002_gb300 import workloads as W
+from tests.helpers import problem
+from tests.test_gpu_fp32bulk import TOL32, _l2, _storage_bound
+
 pytestmark = pytest.mark.gpu
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
@@ -108,3 +112,32 @@ s.close()
 """)
     for k in ("1", "4"):
         assert np.array_equal(r["plain_" + k], r["tight_" + k]), k
+
+
+def test_fp32bulk_without_room_for_the_line_kernels(orc, dg, wrapped, tmp_path):
+    """p = 5: the tiles' face records take more than the one-node kernels'.  The right-hand side is held
+    to the oracle as that of any FP32-bulk context, eight steps to the mode's accuracy target against the
+    context with line kernels."""
+    n, p = 71, 5
+    size = (n * n + 4) // 5 * 4 * 3 * 32 * 4 * 4  # floats of the tiles' face records, in bytes
+    assert size > 12 * 4 * (p + 1) * n * n * 4
+    r = _both(wrapped, tmp_path, size, f"""
+wl = W.drop_2d({n}, {p})
+s = dg.Solver(wl, precision="fp32bulk")
+out[tag + "_lines"] = s.dg_line_kernels(8)
+w = torch.from_numpy(wl.w.copy()).cuda()
+out[tag + "_rhs"] = s.dg_rhs(w).cpu().numpy()
+s.dg_step(w, wl.dt, 8)
+out[tag + "_w"] = w.cpu().numpy()
+assert s.dg_status_read() == 0
+s.close()
+""")
+    assert (r["plain_lines"], r["tight_lines"]) == (1, 0)
+    wl = W.drop_2d(n, p)
+    pb = problem(orc, wl)
+    L_ref, S = orc.rhs(pb, wl.w, want_scale=True)
+    extra = _storage_bound(orc, wl, wl.w)
+    for v in range(7):
+        assert np.abs(r["tight_rhs"][v] - L_ref[v]).max() <= TOL32 * S[v].max() + extra.get(v, 0.0), v
+    assert _l2(r["tight_w"][0], r["plain_w"][0]) <= 1e-5
+    assert _l2(orc.primitives(pb, r["tight_w"])[3], orc.primitives(pb, r["plain_w"])[3]) <= 1e-5
