@@ -30,11 +30,12 @@
  *     asynchronous on that stream unless stated otherwise.  Launch-time
  *     errors are returned; conditions the GPU detects (non-finite values)
  *     are latched in a device status word and reported by dg_status_read.
- *     The FP64 right-hand side's kernels and the FP32-bulk kernels of a grid
- *     that fits on the GPU at once run as programmatic dependent launches; the
- *     latter let the kernel after them on the stream be scheduled early: a
- *     caller's kernel launched with
- *     programmatic stream serialization must call
+ *     The kernels of the FP64 right-hand side, of the adjoint, of the kinematic
+ *     mode on rectangles and of the re-initialisation, and the FP32-bulk kernels
+ *     of a grid that fits on the GPU at once, run as programmatic dependent
+ *     launches; some of the latter let the kernel after them on the stream be
+ *     scheduled early: a caller's kernel launched with programmatic stream
+ *     serialization must call
  *     cudaGridDependencySynchronize() before it reads their results, as
  *     CUDA requires of any such launch.  Ordinary launches, copies and
  *     events on the stream are ordered as usual.
@@ -415,7 +416,7 @@ dg_status dg_kin_step(dg_ctx *ctx, double *w, double t0, double dt, int nsteps, 
    width.  The paper applies ~50 iterations every 2000 steps.  FP64; works on
    FP64 and FP32-bulk contexts alike (on the FP64 state).  The first call
    allocates the context's re-initialisation workspace (3 N doubles and two
-   sets of face traces), kept until dg_destroy.  Rectangles only: a triangle context
+   sets of face traces, one where two do not fit), kept until dg_destroy.  Rectangles only: a triangle context
    gives DG_ERR_UNSUPPORTED.  Asynchronous on stream. */
 dg_status dg_reinit(dg_ctx *ctx, double *w, int niter, double nu, double dtau, void *stream);
 

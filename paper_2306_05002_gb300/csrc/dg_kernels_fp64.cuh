@@ -46,10 +46,10 @@ struct Geom {
   static constexpr int NF = 2 * DIM;                 // faces per element
   static constexpr int NK = DIM == 2 ? P1 : 1;       // nodes per face
   static constexpr int NFK = NF * NK;                // face nodes per element
-  // Elements per block: the smallest count that fills at least 60 threads with
-  // under 7% of the last warp idle.  Small blocks spread a grid evenly over the
-  // 152 SMs (the FP64 path is bound by the per-SM FP64 pipe, so balance, not
-  // occupancy, decides its time).
+  // Elements per block of the FP32-bulk kernels with one node per thread and of
+  // k_ri_sign (the other FP64 kernels choose at launch, pick_epb64; the batched
+  // kernels give EPBX): the smallest count that fills at least 60 threads with
+  // under 7% of the last warp idle.  Small blocks spread a grid evenly over the SMs.
   static constexpr int pick_epb() {
     for (int e = 1; e <= 64; ++e) {
       const int t = e * NP, tp = ((t + 31) / 32) * 32;
@@ -59,7 +59,6 @@ struct Geom {
   }
   static constexpr int EPB = EPBX > 0 ? EPBX : pick_epb();
   static constexpr int THREADS = ((EPB * NP + 31) / 32) * 32;
-  static constexpr int NT = VISC ? NT_VISCOUS : NT_INVISCID;
   static constexpr int NSTAGE = 12;                  // staged fields per node
   static constexpr int OPS = 4 * P1 * P1 + 3 * P1 + NP;  // operator table (OpsLayout) up to cf()
 };

@@ -15,18 +15,22 @@
 //     warp is one run of consecutive 128-, 64- or 32-bit words, and padding lanes have slots of
 //     their own.
 //   * the face records and the volume part are all requested before the first flux is formed.
-// It executes less than half of the instructions per node of the one-node-per-thread kernels (p = 4,
+// It executes half of the thread instructions per node of the one-node-per-thread kernels (p = 4,
 // viscous, surface tension: 780 instead of 1,560; no index arithmetic or divisions per face node, no
 // shared load per term), which is what bounds those on grids of many waves, but a thread's chain is
 // P + 1 times as long and a warp holds four to six times the nodes, so a mesh that does not fill the
 // GPU, and a call too short for its ends, is left to the one-node-per-thread kernels (use_lines32).
-// Measured, 10 steps of a viscous Rayleigh-Taylor problem with surface tension, 256 x 256, p = 4: 3082 us one
-// node per thread, 2795 here.  What bounds them is instruction issue with exposed load latency, at 12 warps
-// an SM.
+// Measured, 10 steps of a viscous Rayleigh-Taylor problem with surface tension, 256 x 256, p = 4: 3089 us one
+// node per thread, 2820 to 2840 here.  What bounds them is instruction issue with exposed load latency, at 12
+// warps an SM.
 //
-// Every operation is rounded as in the one-node-per-thread kernels (see face_flux32), so that the same
-// problem does not change its result with its size class.  Grouping the momentum and energy terms saves
-// another 2%, but turns last bits of the FP32-rounded phase field, 9e-8 at single nodes after four steps.
+// The terms are grouped as in the one-node-per-thread kernels; how the compiler contracts them differs in
+// places.  On periodic meshes (p = 1 to 5, with and without each term) the right-hand side's rows of phi and
+// psi came out the same bits in both, the others within 4e-7 of a row's largest value (7e-6 where its terms
+// cancel: FP32 rounding of them), the state after four steps within 7e-9.  Grouping the
+// momentum and energy terms for fewer operations brings 1.12 instead of 1.10 times
+// on the problem above (1.09 instead of 1.04 on a batch of 32), but turns last bits of the FP32-rounded phase
+// field, 9e-8 at single nodes after four steps.
 // Batches keep one node per thread: on these kernels the mixed ensembles measured 7 to 15% slower, and
 // small ones up to twice as slow.
 #pragma once
@@ -353,9 +357,9 @@ __device__ __forceinline__ Side32 side_of(const LineParams &pf, const float *T) 
 // Strong-form surface integrand F- - F^ of the seven equations at one face node (outward normal sign
 // SG along x, XF, or y) and the lifting coefficients of the symmetric SIP term.  wf: the face weight.
 // tm, tp: own and neighbour records; wall: the ghost side is formed here.
-// Every operation is rounded as in the one-node-per-thread kernels: the right-hand side reads the
-// phase field rounded to FP32, where another rounding anywhere turns single nodes' last bit within a
-// few steps, and the faces amplify that to several units.
+// The terms keep the one-node-per-thread kernels' grouping: the right-hand side reads the phase field
+// rounded to FP32, where another grouping turns single nodes' last bit within a few steps, and the
+// faces amplify that to several units.
 template <bool VISC, bool XF, int SGI>
 __device__ __forceinline__ void face_flux32(const LineParams &pf, const float *tm, float *tp, bool wall, float wf,
                                             float *S, float *lift) {
@@ -1042,10 +1046,13 @@ __device__ __forceinline__ void surface32_tile(const LineParams &pf, float *sm, 
 // Kernels of one problem
 // ---------------------------------------------------------------------------
 constexpr int WPB32 = 2;  // warps per block
-// Blocks per SM asked of the compiler for the stage kernel (register caps of 128, 168, 168 and 204 or 255
-// a thread).  Microseconds a step: p = 3 at 160 x 160, 168 registers 51, 144 57, 128 59; p = 4 viscous at
-// 256 x 256, 207 registers 301, 168 271, 144 313 (spills); p = 5 at 128 x 128, 204 registers 83, 255 96,
-// and viscous, where 204 spill, at 96 x 96 75 and 69.
+// Blocks per SM asked of the compiler for the stage kernel.  An SM's four schedulers hold 16,384 registers
+// each, so the caps are 128 a thread at p <= 2 (spilling up to 80 bytes), 168 at p = 3 and 4 (p = 4 spills 44
+// bytes with viscous stress and surface tension, 36 with surface tension, 24 with viscous stress, none without),
+// 168 at p = 5 (ten warps are three on one scheduler; 136 bytes spilled) and 255 there with any term (254 used).
+// Microseconds a step when these were chosen: p = 3 at 160 x 160, 168 registers 51, 144 57, 128 59; p = 4 with
+// all terms at 256 x 256, uncapped (207) 301, 168 271, 144 313; p = 5 at 128 x 128, five blocks asked 83, four
+// (255) 96, and with all terms at 96 x 96 75 and 69.
 template <int P, bool FULL>
 constexpr int LINE_MINB = P <= 2 ? 8 : P <= 4 ? 6 : FULL ? 4 : 5;
 

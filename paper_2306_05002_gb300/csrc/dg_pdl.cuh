@@ -1,5 +1,7 @@
-// dg_pdl.cuh -- programmatic dependent launch for the FP32-bulk stage kernels
-// of libdgpf (GB300, sm_103a).
+// dg_pdl.cuh -- programmatic dependent launch for the kernels of libdgpf
+// (GB300, sm_103a): the FP32-bulk kernels of grids that fit on the GPU at once,
+// the FP64 right-hand side's, the adjoint's, and those of the kinematic mode on
+// rectangles and of the re-initialisation.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -15,7 +17,8 @@ namespace dgpf {
 // that kernel's tail.  Before its first access to memory that an earlier
 // kernel reads or writes, every thread calls grid_dependency_wait(), which
 // returns once the earlier kernel has completed and its writes are visible.
-// grid_dependents_launch() lets the next kernel be scheduled early.  Both are
+// grid_dependents_launch() lets the next kernel be scheduled early; only the
+// FP32-bulk kernels with one node per thread call it.  Both are
 // no-ops in a kernel launched without the attribute.  Data that an earlier
 // kernel writes is read with coherent loads (ld.global.ca, __ldca), never with
 // the non-coherent ld.global.nc (__ldg): that form declares the data read-only
