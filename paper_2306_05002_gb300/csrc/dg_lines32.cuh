@@ -185,7 +185,7 @@ inline LineUse use_lines32(int P1, bool viscous, bool tension, int E, const Kern
     if (w < 15) return {false, 0};
     const bool rhs = w >= 24;
     if (!viscous) return {rhs, E > one.resident_stage() ? 1 : 0};
-    return {rhs, w >= 50 ? 1 : w >= 30 ? 2 : w >= 21 ? 4 : 6};
+    return {rhs, w >= 50 ? 1 : w >= 30 ? 2 : w >= 24 ? 3 : w >= 21 ? 4 : 6};
   }
   if (w < 50) return {false, 0};
   const bool full5 = P1 == 6 && (viscous || tension), few5 = P1 == 6 && w < 60;
@@ -193,13 +193,13 @@ inline LineUse use_lines32(int P1, bool viscous, bool tension, int E, const Kern
   LineUse u{!few5 && tiles <= (viscous || P1 == 6 ? line.resident_ends() : wave), 0};
   if (E <= one.resident_stage()) return u;
   if (tiles <= wave) {
-    u.steps = P1 < 6 || (full5 && !few5) ? 1 : few5 && !full5 ? 0 : 5;
+    u.steps = P1 < 6 || (full5 && !few5) ? 1 : few5 && !full5 ? 0 : 4;
     return u;
   }
   // percent of the second wave that has to be there; in later ones it matters no more
   const int least = P1 == 4 && (viscous || tension) ? 60 : 35;
   if (full5 || (tiles <= 2 * wave && 100 * (tiles - wave) < least * wave)) return u;
-  u.steps = P1 == 6 || (P1 == 4 && viscous) ? 5 : viscous ? 3 : 2;
+  u.steps = P1 == 6 ? 4 : !viscous ? 2 : P1 == 4 ? 5 : 3;
   return u;
 }
 
